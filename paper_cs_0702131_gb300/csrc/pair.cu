@@ -25,7 +25,9 @@
 // flag_ill_conditioned and refine_ds recompute in double-single arithmetic
 // the molecules whose FP32 force the error bound cannot certify.  The cell
 // kernel pair_fwd32 described next serves general referring transforms, the
-// vertex criterion and AICA_OPT_FP32_KERNEL = 1; pair_fwd64 is the FP64 path.
+// vertex criterion and AICA_OPT_FP32_KERNEL = 1.  FP64 forces and adjoint run
+// over clusters too (pair64.cu); pair_fwd64 and pair_bwd64 here serve general
+// transforms, the vertex criterion and (forces) portion mode.
 //
 // FP32 cell kernel layout.  A persistent grid of 4-warp blocks; warps claim
 // cells from a global counter.  The chunk (up to NI molecules of I: 4 for cells of a
@@ -60,68 +62,15 @@
 #include <algorithm>
 
 #include "aica_internal.cuh"
+#include "pair_common.cuh"
 
 namespace aica {
 namespace {
 
 constexpr int kPairThreads = 256;
 constexpr int kWarps = kPairThreads / 32;
-constexpr int kParts = 16;           // accumulator row: U, W[6], counters[8]
 constexpr int NI = 8;                // i-molecules per chunk in the FP64 kernel
 
-struct SpeciesTab {
-    float4 f[kMaxSpecies * kMaxSpecies];    // sigma^2, 24 eps, 4 eps, u(rc) for FP32
-    double d[kMaxSpecies * kMaxSpecies][4]; // same in FP64
-};
-
-struct PairArgs {
-    int C;
-    const int *cell_off, *work_off;
-    const WorkEntry *work;
-    const int *run_off;
-    const RunEntry *runs;
-    const int *orgm;             // molecule-frame origins in units of 2^-10
-    float Lhi[3], Llo[3];        // box lengths as float pairs (Lhi + Llo = L to ~1e-14)
-    const float4 *xloc;
-    const double *xs64;
-    const float4 *sph;           // per-cell molecule bounding spheres (local frame)
-    float rc2_lo, rc2_hi;
-    float rc2_pre;               // cluster kernel: hi-part test threshold (margin above the remainders)
-    double rc2_d;
-    double L[3];
-    int S;
-    void *facc;                  // float4 (FP32) or double4 (FP64), binned order
-    const void *vs;              // backward: grad_force in binned order (float4 / double4)
-    double *acc;                 // [0..6] U, W; [8..15] counters (as unsigned long long); [16..] grads
-    unsigned *next_cell;         // FP32 kernel: next unclaimed cell (zero at launch)
-    int ghosts;                  // portion mode: xloc.w carries kGhostBit on halo molecules
-    int xf;                      // general referring transforms: image field = transform index
-    int n_xf;                    // transforms in xft
-    const XfDev *xft;            // [n_xf] transforms (identity first)
-    const float4 *run_d;         // general transforms: shift of each run in I's molecule frame
-    SpeciesTab tab;
-};
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-template <class R> struct R3 { R x, y, z; };
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// FP64 re-decision of r^2 < rc^2 with the all-pairs definition's operation order
 // image y_t + R_t x of x under referring transform t, in the oracle's operation order
 __device__ __forceinline__ void xf_image(const XfDev &t, const double *x, double *q) {
     for (int i = 0; i < 3; ++i)
@@ -138,32 +87,6 @@ __device__ __noinline__ bool band_in_xf(const PairArgs &a, int k, int l, int np)
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)) < a.rc2_d;
 }
 
-__device__ __noinline__ bool band_in(const PairArgs &a, int k, int l, int np) {
-    const double *xk = a.xs64 + 3 * (size_t)k, *xl = a.xs64 + 3 * (size_t)l;
-    double dx = __dsub_rn(__dsub_rn(xk[0], xl[0]), __dmul_rn(a.L[0], (double)unpack_n(np, 0)));
-    double dy = __dsub_rn(__dsub_rn(xk[1], xl[1]), __dmul_rn(a.L[1], (double)unpack_n(np, 1)));
-    double dz = __dsub_rn(__dsub_rn(xk[2], xl[2]), __dmul_rn(a.L[2], (double)unpack_n(np, 2)));
-    double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    return r2 < a.rc2_d;
-}
-
-// Sums of the pair kernels.  Every warp adds its totals (FP64 sums identical
-// in all lanes; counters per lane) to one of kStripes rows of FP64
-// accumulators (row = warp index mod kStripes, so few warps share an
-// address); finish_sums adds the rows.  Row layout: [0..6] U and W,
-// [7..14] the counters, exactly representable in FP64.
-constexpr int kStripes = 64;
-constexpr int kAccStripes = 64;        // offset of the rows in acc (doubles)
-
-__device__ void warp_to_stripe(const PairArgs &a, int gwarp, const double (&dsum)[7], const unsigned (&cv)[8],
-                               int lane) {
-    double *row = a.acc + kAccStripes + (size_t)(gwarp % kStripes) * kParts;
-    for (int i = 0; i < 8; ++i) {
-        const unsigned s = __reduce_add_sync(0xffffffffu, cv[i]);
-        if (lane == 0 && s) atomicAdd(row + 7 + i, (double)s);
-    }
-    if (lane < 7) atomicAdd(row + lane, dsum[lane < 7 ? lane : 0]);
-}
 
 // Totals of the stripe rows into acc ([0..6] FP64, [8..15] counters as
 // unsigned 64-bit) and the caller's energy/virial [7] and pair counts [6].
@@ -636,21 +559,6 @@ __device__ __forceinline__ void pair64(const double (*tab)[4], double rx, double
     acc[4] += w * (rx * fy); acc[5] += w * (rx * fz); acc[6] += w * (ry * fz);
 }
 
-__device__ __forceinline__ void atomic_add3(double *p, double x, double y, double z) {
-    atomicAdd(p, x);
-    atomicAdd(p + 1, y);
-    atomicAdd(p + 2, z);
-}
-
-// r = (x_k - x_l) - n.L with the all-pairs definition's rounding
-__device__ __forceinline__ void sep64(const double *xk, const double *xl, const double *L, int np, double &rx,
-                                      double &ry, double &rz, double &r2) {
-    rx = __dsub_rn(__dsub_rn(xk[0], xl[0]), __dmul_rn(L[0], (double)unpack_n(np, 0)));
-    ry = __dsub_rn(__dsub_rn(xk[1], xl[1]), __dmul_rn(L[1], (double)unpack_n(np, 1)));
-    rz = __dsub_rn(__dsub_rn(xk[2], xl[2]), __dmul_rn(L[2], (double)unpack_n(np, 2)));
-    r2 = __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
-}
-
 // r = x_k - (y_t + R_t x_l) under referring transform t (general transforms), else sep64
 template <bool XF>
 __device__ __forceinline__ void sep64x(const PairArgs &a, const double *xk, const double *xl, int np, double &rx,
@@ -901,17 +809,6 @@ __global__ void __launch_bounds__(256) unsort_forces(const int *inv, int64_t n, 
     out[3 * k] = (T)x;
     out[3 * k + 1] = (T)y;
     out[3 * k + 2] = (T)z;
-}
-
-// A binned molecule split at multiples of 2^-q: hi exact on the grid, lo the
-// rest (xloc - hi is exact; adding the stored remainder rounds far below
-// the separation's own rounding).  Valid for |x| < 2^(22 - q).
-__device__ __forceinline__ void grid_split(float4 x, float4 r, float qr, float4 &hi, float4 &lo) {
-    hi.x = __fsub_rn(__fadd_rn(x.x, qr), qr);
-    hi.y = __fsub_rn(__fadd_rn(x.y, qr), qr);
-    hi.z = __fsub_rn(__fadd_rn(x.z, qr), qr);
-    hi.w = x.w;
-    lo = make_float4(__fsub_rn(x.x, hi.x) + r.x, __fsub_rn(x.y, hi.y) + r.y, __fsub_rn(x.z, hi.z) + r.z, 0.f);
 }
 
 // The FP32 error of a molecule's force is about a fixed multiple of
@@ -1230,13 +1127,6 @@ __global__ void __launch_bounds__(256) refine_ds(PairArgs a, RefineArgs r) {
 // Species sums: slots [0, 8) hold dL/d eps_s and [8, 16) dL/d sigma_s; each
 // warp adds its totals to the striped FP64 rows of the forward kernels, and
 // finish_bwd adds the rows.
-constexpr int kGradSlots = 2 * kMaxSpecies;
-static_assert(kGradSlots <= kParts, "gradient slots must fit a stripe row");
-
-struct BwdTab {
-    double eps, sig2, inv_eps, inv_sig, fa, fb;   // fa, fb: d eps_ab / d eps_a, d eps_ab / d eps_b
-};
-
 struct BwdArgs {
     PairArgs p;
     BwdTab t[kMaxSpecies * kMaxSpecies];
@@ -1244,12 +1134,6 @@ struct BwdArgs {
     double e1, s1;                          // one species: 1 / eps, 1 / sigma
     int S;
 };
-
-// A warp's species-gradient totals (lane q < kGradSlots holds slot q) into its stripe row.
-__device__ __forceinline__ void grads_to_stripe(const PairArgs &a, int gwarp, double g, int lane) {
-    double *row = a.acc + kAccStripes + (size_t)(gwarp % kStripes) * kParts;
-    if (lane < kGradSlots && g != 0.0) atomicAdd(row + lane, g);
-}
 
 // R^T g for a row-major FP32 rotation R
 __device__ __forceinline__ float3 rot32t(const float *R, float x, float y, float z) {
@@ -1642,16 +1526,6 @@ __global__ void __launch_bounds__(kGradSlots * 32) finish_bwd(const double *acc,
 // Every force accumulator's .w sums |f|^2 over the molecule's pairs: the
 // scale of the FP32 error of its force (see flag_ill_conditioned and
 // refine_ds).
-struct ClKArgs {
-    const int *cl_first, *cl_run_off;
-    const ClRun *runs;
-    const float4 *xlo;
-    float4 *cl_box;              // out: each cluster's box of molecules (lo, hi; hi parts, own frame)
-    int ncl;
-    float qround;                // 1.5 * 2^(23 - q): x + qround - qround rounds x to a multiple of 2^-q
-};
-
-
 constexpr int kCT = 128, kCW = kCT / 32;
 // A molecule's FP32 force error is about a multiple of sqrt(sum_l |f_kl|^2)
 // (rounding of each pair force, mostly; the separations are rounded once);
@@ -1660,14 +1534,6 @@ constexpr int kCT = 128, kCW = kCT / 32;
 constexpr double kRefineScale = 1.25e-6;
 constexpr int kCap = 176;                 // survivors buffered per warp (5 blocks of 4 warps per SM)
 constexpr int kNI = 8;                    // molecules of A per i-tile
-// packed survivor / tile word (.w of the hi position)
-constexpr int kSpBits = 7, kSameBit = 1 << 3, kImgBit = 1 << 4, kGhostW = 1 << 21;
-__device__ __forceinline__ int cellq_of(int w) { return (w >> 5) & 15; }
-__device__ __forceinline__ int32_t n_of(int w) {   // 3 x 4-bit image -> pack_n
-    const int c = w >> 9;
-    return pack_n((c << 28) >> 28, (c << 24) >> 28, (c << 20) >> 28);
-}
-
 struct WarpC {
     float4 sh[kCap];      // survivor: position in A's frame, hi part (exact); .w packed word
     float4 sl[kCap];      // survivor: remainder (xyz); .w binned index (int bits)
@@ -2208,6 +2074,18 @@ void fill_common(aica_mesh *m, PairArgs &a) {
     a.ghosts = m->ghosts ? 1 : 0;
 }
 
+ClKArgs cluster_args(aica_mesh *m) {
+    ClKArgs c{};
+    c.cl_first = m->cl_first.as<int>();
+    c.cl_run_off = m->cl_run_off.as<int>();
+    c.runs = m->cl_runs.as<ClRun>();
+    c.xlo = m->xlo.as<float4>();
+    c.cl_box = m->cl_box.as<float4>();
+    c.ncl = (int)m->n_cl;
+    c.qround = (float)ldexp(1.5, 23 - m->qexp);
+    return c;
+}
+
 aica_status check_flags(aica_mesh *m, cudaStream_t st) {
     unsigned flags = 0;
     AICA_CUDA(cudaMemcpyAsync(&flags, m->flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
@@ -2360,8 +2238,8 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
     AICA_CUDA(timing_begin(m, st, &tstop));
     // FP32 with box periodicity: the cluster kernel when the lists have a
     // cluster schedule (the cell kernel on request, and for general transforms)
-    const bool clsched = !f64 && !a.xf && m->n_cl_runs >= 0;
-    const bool clpath = clsched && m->fp32_kernel != 1;
+    const bool clsched = !a.xf && m->n_cl_runs >= 0;
+    const bool clpath = clsched && !f64 && m->fp32_kernel != 1;
     if (m->ghosts && !f64 && !clpath) {
         set_error("aica_forces: portion mode (halo molecules) needs the FP32 cluster kernel");
         return AICA_ERR_INVALID_ARG;
@@ -2370,16 +2248,10 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
         set_error("aica_forces: portion mode (halo molecules) needs box periodicity");
         return AICA_ERR_INVALID_ARG;
     }
+    const ClKArgs c = cluster_args(m);
+    bool cl64 = false;                 // FP64 cluster kernel
     if (!f64) {
         if (clpath) {
-            ClKArgs c{};
-            c.cl_first = m->cl_first.as<int>();
-            c.cl_run_off = m->cl_run_off.as<int>();
-            c.runs = m->cl_runs.as<ClRun>();
-            c.xlo = m->xlo.as<float4>();
-            c.cl_box = m->cl_box.as<float4>();
-            c.ncl = (int)m->n_cl;
-            c.qround = (float)ldexp(1.5, 23 - m->qexp);
             launch_fwd32c(a, c, multi, shift, st);
         } else {
             // i-chunk width: 4 for cells of a few molecules (tetrahedra), 8 otherwise
@@ -2387,14 +2259,16 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
             else launch_fwd32<8>(a, multi, shift, st);
         }
     } else {
-        if (a.xf) launch_fwd64<true>(a, multi, shift, grid, st);
+        cl64 = clsched && !m->ghosts && launch_fwd64c(a, c, lj, st);
+        if (cl64) {
+        } else if (a.xf) launch_fwd64<true>(a, multi, shift, grid, st);
         else launch_fwd64<false>(a, multi, shift, grid, st);
     }
     AICA_CUDA(timing_end(tstop, st));
     m->launches = 2;
     double *acc = m->acc.as<double>();
-    if (clpath && counts_out && m->count_evaluated && a.C > 0) {
-        // the cluster kernel does not walk the cell schedule: count the method's evaluated pairs
+    if (counts_out && a.C > 0 && ((clpath && m->count_evaluated) || cl64)) {
+        // the cluster kernels do not walk the cell schedule: count the method's evaluated pairs
         count_evaluated<<<(unsigned)std::min<int64_t>(((int64_t)a.C * 32 + 255) / 256, 152 * 16), 256, 0, st>>>(
             a.cell_off, a.run_off, a.runs, a.C, acc);
         m->launches += 1;
@@ -2513,7 +2387,8 @@ extern "C" aica_status aica_forces_backward(aica_mesh *m, const aica_lj *lj, aic
     cudaEvent_t tstop;
     AICA_CUDA(timing_begin(m, st, &tstop));
     if (f64) {
-        launch_bwd64(b, multi, pair_grid(b.p.C), st);
+        const bool clsched = !b.p.xf && m->n_cl_runs >= 0;
+        if (!(clsched && launch_bwd64c(b.p, cluster_args(m), lj, b.t, st))) launch_bwd64(b, multi, pair_grid(b.p.C), st);
     } else {
         if ((double)n < 5.0 * (double)b.p.C) launch_bwd32<4>(b, multi, st);
         else launch_bwd32<8>(b, multi, st);
