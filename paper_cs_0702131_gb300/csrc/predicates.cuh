@@ -118,6 +118,15 @@ static __host__ __device__ __noinline__ int exact_det3_sign(const double *a, con
 
 // exact sign of (b_i - a_i)(c_j - a_j) - (b_j - a_j)(c_i - a_i)
 static __device__ __noinline__ int exact_det2_sign(const double *a, const double *b, const double *c, int i, int j) {
+    {
+        // FP64 first: differences and products carry a few 2^-53 of their
+        // magnitude each; both products exactly zero decide too
+        const double x = b[i] - a[i], y = c[j] - a[j], z = b[j] - a[j], t = c[i] - a[i];
+        const double p = x * y, q = z * t, perm = fabs(p) + fabs(q), det = p - q;
+        if (det > 1e-14 * perm) return 1;
+        if (det < -1e-14 * perm) return -1;
+        if ((x == 0.0 || y == 0.0) && (z == 0.0 || t == 0.0)) return 0;
+    }
     double x[2], y[2], z[2], t[2];
     two_diff(b[i], a[i], x[0], x[1]);
     two_diff(c[j], a[j], y[0], y[1]);
@@ -158,6 +167,9 @@ static __device__ __noinline__ int orient_sos_slow(const double *a, const double
     int s;
     if (det > 1e-14 * perm) s = 1;
     else if (det < -1e-14 * perm) s = -1;
+    else if ((u[0] == 0.0 && v[0] == 0.0 && w[0] == 0.0) || (u[1] == 0.0 && v[1] == 0.0 && w[1] == 0.0) ||
+             (u[2] == 0.0 && v[2] == 0.0 && w[2] == 0.0))
+        s = 0;               // p on the triangle's axis-aligned plane (walls on lattice planes): exactly zero
     else s = exact_det3_sign(a, b, c, p);
     if (s != 0) return -s;   // O = -det[a-p; b-p; c-p]
     // p on the plane: N_x, N_y, N_z of N = (b - a) x (c - a), exactly
