@@ -117,6 +117,13 @@ __host__ __device__ inline int unpack_n(int32_t p, int axis) {
     return (int)(signed char)((p >> (8 * axis)) & 0xff);
 }
 
+// Whether words cleared by this call's own memset may count as clean for later
+// calls: not when the memset was only captured into a graph.
+inline bool really_ran(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+}
+
 }  // namespace aica
 
 struct aica_mesh;
@@ -213,6 +220,17 @@ struct aica_mesh {
     aica::DevBuf flags;                      // unsigned[4] device error flags
     aica::DevBuf params;                     // per-call parameter block
     aica::DevBuf tmp;                        // general scratch
+
+    // Words that the kernels of a call leave zero for the next one, so that no
+    // call clears them first: the cell counts and the miss count (binning), the
+    // force accumulators, the sums, the species word of the flags.  False until
+    // cleared, and again from the start of a call until its launches succeeded.
+    bool bin_clean = false, facc_clean = false, acc_clean = false, flags_clean = false;
+    // Flags of the last checked binning, written by its last block to mapped
+    // host memory (pub; NULL if there is none).
+    unsigned *pub = nullptr, *pub_dev = nullptr;
+    bool pub_valid = false;                  // pub_flags are the device's error bits
+    unsigned pub_flags = 0;
 
     bool deferred = false;
     int64_t launches = 0;

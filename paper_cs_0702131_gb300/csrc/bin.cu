@@ -79,7 +79,8 @@ struct BinArgs {
     int *cell_of;
     int *cnt;              // molecules per cell (counted as they are located)
     int *inv;              // original -> binned index; -1 for molecules in no cell
-    unsigned *flags;
+    unsigned *flags;       // [0] error bits, [1] largest species index, [2] blocks that are done
+    unsigned *pub;         // host: flags[0], flags[1] of this call (checked calls; NULL: not written)
 };
 
 // Add one molecule to cell c's count (c < 0: none), aggregated over the warp's
@@ -591,6 +592,21 @@ __device__ __forceinline__ void frame_split(const BinArgs &a, const double *p, c
 // coordinates local to the cell's molecule-frame origin into binned order, record the
 // inverse permutation, and the cell's bounding sphere (centre = mean, radius
 // = largest distance, rounded up) that the pair kernels cull with.
+// End of a binning's last kernel: its last block hands the flags to the host
+// (instead of a copy after it) and leaves the species word zero.
+__device__ __forceinline__ void publish_flags(const BinArgs &a) {
+    if (!a.pub) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(a.flags + 2, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    a.pub[0] = atomicAdd(a.flags, 0u);
+    a.pub[1] = atomicExch(a.flags + 1, 0u);
+    a.flags[2] = 0;
+    __threadfence_system();
+}
+
 template <int G>
 __global__ void __launch_bounds__(256) bin_cells(BinArgs a, const int *cell_off, int C, int *order, double *xs64,
                                                  float4 *xloc, float4 *sph) {
@@ -690,6 +706,7 @@ __global__ void __launch_bounds__(256) bin_cells(BinArgs a, const int *cell_off,
     const int mx = __reduce_max_sync(0xffffffffu, spmax);
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.flags, kFlagSpecies);
     if (lane == 0 && mx > 0) atomicMax((int *)a.flags + 1, mx);
+    publish_flags(a);
 }
 
 // The same per slot, for cells of a few molecules.  Warp w owns the cells
@@ -744,9 +761,8 @@ __device__ __forceinline__ float4 sphere_of(const float4 *x, int m) {
     return make_float4(cx, cy, cz, sqrtf(rr) * (1.f + 1e-5f) + 1e-5f);
 }
 
-__global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const int *cell_off, const int *nbp,
-                                                             const int *un, const int *ucell, int *order,
-                                                             double *xs64, float4 *xloc, float4 *sph) {
+__device__ __forceinline__ void bin_slots_warp(const BinArgs &a, const int *cell_off, const int *nbp, const int *un,
+                                               const int *ucell, int *order, double *xs64, float4 *xloc, float4 *sph) {
     __shared__ int sk[kSlotWarps][64];
     __shared__ float4 sx[kSlotWarps][64];
     const unsigned FULL = 0xffffffffu;
@@ -844,6 +860,13 @@ __global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const in
     if (lane == 0 && mx > 0) atomicMax((int *)a.flags + 1, mx);
 }
 
+__global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const int *cell_off, const int *nbp,
+                                                             const int *un, const int *ucell, int *order,
+                                                             double *xs64, float4 *xloc, float4 *sph) {
+    bin_slots_warp(a, cell_off, nbp, un, ucell, order, xs64, xloc, sph);
+    publish_flags(a);
+}
+
 }  // namespace
 }  // namespace aica
 
@@ -862,7 +885,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->launches = 0;
     m->binned = false;
     if (n > m->cap_mol) {
-        m->hint_valid = false;
+        m->hint_valid = m->facc_clean = false;
         int64_t cap = std::max<int64_t>(n, 1024);
         AICA_CUDA(m->cell_of.reserve(sizeof(int) * cap));
         AICA_CUDA(m->order.reserve(sizeof(int) * cap));
@@ -878,9 +901,11 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
         m->cap_mol = cap;
     }
     AICA_CUDA(m->cell_off.reserve(sizeof(int) * (C + 1)));
+    const void *old_fill = m->fill.p, *old_miss = m->miss.p;
     AICA_CUDA(m->fill.reserve(sizeof(int) * (C + 1)));
     AICA_CUDA(m->sph.reserve(sizeof(float4) * C));
     AICA_CUDA(m->miss.reserve(sizeof(int) * (std::max<int64_t>(n, 1) + 1)));
+    if (m->fill.p != old_fill || m->miss.p != old_miss) m->bin_clean = false;
     m->n_mol = n;
     BinArgs a{};
     a.n = n;
@@ -940,15 +965,22 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     int *off = m->cell_off.as<int>();
     a.cnt = cnt;
     a.inv = m->inv.as<int>();
-    // with deferred checks the error bits (flags[0]) accumulate until aica_check_status
-    if (m->deferred) AICA_CUDA(cudaMemsetAsync(m->flags.as<unsigned>() + 1, 0, 12, st));
-    else AICA_CUDA(cudaMemsetAsync(m->flags.p, 0, 16, st));
-    AICA_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (C + 1), st));
+    // with deferred checks the error bits (flags[0]) accumulate until
+    // aica_check_status; a checked call's last kernel hands them to the host
+    const bool publish = !m->deferred && m->pub && n > 0 && C > 0;
+    a.pub = publish ? m->pub_dev : nullptr;
+    if (!m->deferred && !m->flags_clean) AICA_CUDA(cudaMemsetAsync(m->flags.p, 0, 16, st));
+    m->flags_clean = m->pub_valid = false;
+    const bool was_clean = m->bin_clean;
+    if (!was_clean) {
+        AICA_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (C + 1), st));
+        AICA_CUDA(cudaMemsetAsync(m->miss.p, 0, sizeof(int), st));
+    }
+    m->bin_clean = false;
     unsigned nb = (unsigned)((n + 255) / 256);
     if (n > 0) {
         // locate every molecule and count the cells' molecules
         if (a.hint) {
-            AICA_CUDA(cudaMemsetAsync(m->miss.p, 0, sizeof(int), st));
             // small systems: small blocks, so that every SM has some of the (latency-bound) warps
             const unsigned lb = n <= 152 * 512 ? 64 : 256;
             bin_locate_hint<<<(unsigned)((n + lb - 1) / lb), lb, 0, st>>>(a);
@@ -960,7 +992,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
         }
     }
     m->launches += exclusive_scan_1pass(cnt, C, off, m->scan_state.as<unsigned long long>(), m->flags.as<unsigned>(),
-                                        kFlagTimeout, st);
+                                        kFlagTimeout, m->miss.as<int>(), st);
     // wide cells are sorted in place in `order`; narrow ones go from `unsorted` to `order`
     const bool wide = (double)n > 6.0 * (double)C;
     int *slots_out = wide ? m->order.as<int>() : m->unsorted.as<int>();
@@ -982,6 +1014,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->n_mol_prev = n;
     m->hint_valid = true;
     AICA_CUDA(cudaGetLastError());
+    m->bin_clean = was_clean || really_ran(st);
     if (cell_of && n) AICA_CUDA(cudaMemcpyAsync(cell_of, a.cell_of, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (order && n) AICA_CUDA(cudaMemcpyAsync(order, m->order.p, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (cell_off) AICA_CUDA(cudaMemcpyAsync(cell_off, off, sizeof(int) * (C + 1), cudaMemcpyDeviceToDevice, st));
@@ -989,8 +1022,16 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->max_species = -1;
     if (!m->deferred) {
         unsigned flags[2] = {0, 0};
-        AICA_CUDA(cudaMemcpyAsync(flags, m->flags.p, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+        if (!publish) AICA_CUDA(cudaMemcpyAsync(flags, m->flags.p, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
         AICA_CUDA(cudaStreamSynchronize(st));
+        if (publish) {
+            flags[0] = ((volatile unsigned *)m->pub)[0];
+            flags[1] = ((volatile unsigned *)m->pub)[1];
+            m->flags_clean = flags[0] == 0;
+            m->pub_valid = true;
+            m->pub_flags = flags[0];
+        }
+        if (flags[0] & kFlagTimeout) m->bin_clean = false;
         m->max_species = (int)flags[1];
         if (flags[0] & kFlagSpecies) {
             set_error("aica_bin_molecules: species index outside [0, %d)", kMaxSpecies);

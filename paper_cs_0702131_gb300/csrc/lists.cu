@@ -732,6 +732,7 @@ extern "C" aica_status aica_build_interaction_list_ex(aica_mesh *m, double rc, d
     m->launches = 0;
     m->built = false;
     m->n_cl_runs = -1;
+    m->flags_clean = m->pub_valid = false;      // the builder uses the flag words
 
     // ---- centroid bucket grid (host): about one cell per bucket
     QArgs a{};

@@ -500,6 +500,12 @@ extern "C" aica_status aica_mesh_create(const double *points, int64_t n_points, 
         aica_mesh_destroy(m);
         return s;
     }
+    if (cudaHostAlloc((void **)&m->pub, 64, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void **)&m->pub_dev, m->pub, 0) != cudaSuccess) {
+        cudaGetLastError();              // without it the flags are copied
+        if (m->pub) cudaFreeHost(m->pub);
+        m->pub = m->pub_dev = nullptr;
+    }
     m->h_ctr.swap(h_ctr);
     m->h_rad.swap(h_rad);
     *out = m;
@@ -513,8 +519,9 @@ extern "C" void aica_mesh_destroy(aica_mesh *m) {
                             &m->dil_ids, &m->ref_src, &m->ref_n, &m->ref_off, &m->ref_ids, &m->run_off, &m->runs, &m->xf_dev, &m->run_d, &m->work_off,
                             &m->work, &m->work_split, &m->proc_order, &m->cell_of, &m->order, &m->unsorted, &m->ucell,
                             &m->cell_off, &m->fill, &m->inv, &m->sph, &m->xloc, &m->xs64, &m->facc,
-                            &m->vsorted, &m->acc, &m->flags, &m->params, &m->tmp, &m->scan_state};
+                            &m->vsorted, &m->acc, &m->flags, &m->params, &m->tmp, &m->scan_state, &m->miss};
     for (auto *b : bufs) b->release();
+    if (m->pub) cudaFreeHost(m->pub);
     for (auto *v : {&m->tev, &m->tfree})
         for (auto &p : *v) {
             cudaEventDestroy(p.first);

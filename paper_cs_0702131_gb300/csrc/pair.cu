@@ -22,7 +22,7 @@
 // Kernels.  With box periodicity and the minimum-distance lists the FP32
 // forces come from the cluster kernel pair_fwd32c (further below: a warp
 // per cluster of cells, candidates culled against the cluster's box), then
-// flag_ill_conditioned and refine_ds recompute in double-single arithmetic
+// finish_forces and refine_ds list and recompute in double-single arithmetic
 // the molecules whose FP32 force the error bound cannot certify.  The cell
 // kernel pair_fwd32 described next serves general referring transforms, the
 // vertex criterion and AICA_OPT_FP32_KERNEL = 1.  FP64 forces and adjoint run
@@ -106,10 +106,19 @@ __device__ __forceinline__ void finish_value(double *acc, double *ev, long long 
     }
 }
 
+// Leave the sums' rows and the unit counters zero for the next call (a whole
+// block, after its finish_value calls).
+__device__ __forceinline__ void clear_sums(double *acc) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < kStripes * kParts; i += blockDim.x) acc[kAccStripes + i] = 0.0;
+    if (threadIdx.x < 2) acc[24 + threadIdx.x] = 0.0;
+}
+
 // One warp per value (15 warps); used when no molecule was binned (otherwise
-// the first block of unsort_forces does it).
+// the first block of finish_forces does it).
 __global__ void __launch_bounds__(15 * 32) finish_sums(double *acc, double *ev, long long *counts) {
     finish_value(acc, ev, counts, threadIdx.x >> 5, threadIdx.x & 31);
+    clear_sums(acc);
 }
 
 // ------------------------------------------------------------------ FP32 path
@@ -781,49 +790,51 @@ __global__ void __launch_bounds__(kPairThreads) pair_fwd64(PairArgs a) {
     warp_to_stripe(a, gwarp, dsum, cv, lane);
 }
 
-// ---------------------------------------------------------------- unsort
-// Forces back to the original order; with acc, the first block also adds
-// up the pair kernel's striped sums (finish_value).
+// ---------------------------------------------------------------- results
+// One pass over the binned molecules (cell_off[C] of them): forces to the
+// original order (rows of molecules in no cell are zero), the totals of the
+// pair kernel's striped sums (acc, in the first block), and the flag list
+// (kflag2 > 0): the FP32 error of a molecule's force is about a fixed multiple of
+// sqrt(sum |f|^2) (the .w of its accumulator); a molecule whose force is too
+// small against it goes to the list for recomputation.  The list follows the
+// binned order (one append per block), so the molecules' positions.
+// Accumulators and sums are left zero for the next call.  Memory-bound and
+// small, so what counts is the launches: this one takes the place of two
+// kernels (256 000 molecules: 6.1 and 4.9 us) and of two memsets per call.
 template <class T>
-__global__ void __launch_bounds__(256) unsort_forces(const int *inv, int64_t n, const void *facc, T *out, int f64,
-                                                     double *acc = nullptr, double *ev = nullptr,
-                                                     long long *counts = nullptr, int *flag_list = nullptr,
-                                                     float kflag2 = 0.f) {
-    if (acc && blockIdx.x == 0)
+__global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C, const int *order, const int *inv,
+                                                     int64_t n, void *facc, T *out, double *acc, double *ev,
+                                                     long long *counts, const float4 *xloc, float kflag2,
+                                                     int *flag_list) {
+    __shared__ int wcnt[8], wbase[8];
+    if (acc && blockIdx.x == 0) {
         for (int i = threadIdx.x >> 5; i < 15; i += blockDim.x >> 5) finish_value(acc, ev, counts, i, threadIdx.x & 31);
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    int s = inv[k];
-    double x = 0, y = 0, z = 0;
-    if (s >= 0) {
-        if (f64) {
-            const double *f = (const double *)facc + 4 * (size_t)s;
-            x = f[0]; y = f[1]; z = f[2];
+        clear_sums(acc);
+    }
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    bool f = false;
+    if (k < n && inv[k] < 0) out[3 * k] = out[3 * k + 1] = out[3 * k + 2] = (T)0;
+    if (k < cell_off[C]) {
+        T *o = out + 3 * (int64_t)order[k];
+        if (sizeof(T) == 8) {
+            double2 *v = (double2 *)facc + 2 * k;
+            const double2 xy = v[0];
+            const double z = v[1].x;
+            v[0] = v[1] = make_double2(0.0, 0.0);
+            o[0] = (T)xy.x;
+            o[1] = (T)xy.y;
+            o[2] = (T)z;
         } else {
-            float4 f = ((const float4 *)facc)[s];
-            x = f.x; y = f.y; z = f.z;
-            (void)flag_list;
-            (void)kflag2;
+            const float4 v = ((float4 *)facc)[k];
+            ((float4 *)facc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            o[0] = (T)v.x;
+            o[1] = (T)v.y;
+            o[2] = (T)v.z;
+            f = kflag2 > 0.f && v.x * v.x + v.y * v.y + v.z * v.z < kflag2 * v.w &&
+                !(__float_as_int(xloc[k].w) & kGhostBit);
         }
     }
-    out[3 * k] = (T)x;
-    out[3 * k + 1] = (T)y;
-    out[3 * k + 2] = (T)z;
-}
-
-// The FP32 error of a molecule's force is about a fixed multiple of
-// sqrt(sum |f|^2) (the .w of its accumulator); a molecule whose force is too
-// small against it goes to the list for recomputation.  In binned order,
-// one append per warp, so the list follows the molecules' positions.
-__global__ void __launch_bounds__(256) flag_ill_conditioned(const float4 *facc, const float4 *xloc, int nb,
-                                                              float kflag2, int *flag_list) {
-    __shared__ int wcnt[8], wbase[8];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    bool f = false;
-    if (s < nb) {
-        const float4 v = facc[s];
-        f = v.x * v.x + v.y * v.y + v.z * v.z < kflag2 * v.w && !(__float_as_int(xloc[s].w) & kGhostBit);
-    }
+    if (!(kflag2 > 0.f)) return;
     const unsigned b = __ballot_sync(0xffffffffu, f);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (lane == 0) wcnt[w] = __popc(b);
@@ -838,7 +849,7 @@ __global__ void __launch_bounds__(256) flag_ill_conditioned(const float4 *facc, 
         for (int i = 0; i < 8; ++i) wbase[i] += base;
     }
     __syncthreads();
-    if (f) flag_list[1 + wbase[w] + __popc(b & ((1u << lane) - 1u))] = s;
+    if (f) flag_list[1 + wbase[w] + __popc(b & ((1u << lane) - 1u))] = (int)k;
 }
 
 // Double-single ("float-float") arithmetic: a value is an unevaluated sum
@@ -876,7 +887,7 @@ __device__ __forceinline__ ds ds_rcp(ds a) {
     return ds_fast2sum(y, __fmul_rn(y, e));
 }
 
-// Recomputation of the molecules flagged by unsort_forces: a warp per
+// Recomputation of the molecules flagged by finish_forces: a warp per
 // molecule k (binned) of cluster A, lanes over the molecules of A and of
 // every (partner cluster, image) of A's full list.  Each separation is
 // formed exactly before one rounding (hi parts on the 2^-q grid, as in the
@@ -1285,10 +1296,13 @@ __global__ void __launch_bounds__(kThreads32, MINB) pair_bwd32(BwdArgs b) {
         }
     };
     int ncell = 0;
-    int I0 = lane == 0 ? (int)atomicAdd(a.next_cell, (unsigned)kGrab) : 0;
-    I0 = __shfl_sync(FULL, I0, 0);
+    // the first cells by warp, the next ones claimed while these are worked on:
+    // with enough warps for all cells the grouping of the species' FP32 sums, so
+    // their last bits, does not depend on the order in which warps start
+    const int nwarps = gridDim.x * kWarps32;
+    int I0 = (blockIdx.x * kWarps32 + wib) * kGrab;
     while (I0 < a.C) {
-        const int Inext = lane == 0 ? (int)atomicAdd(a.next_cell, (unsigned)kGrab) : 0;
+        const int Inext = nwarps * kGrab + (lane == 0 ? (int)atomicAdd(a.next_cell, (unsigned)kGrab) : 0);
         const int Iend = min(I0 + kGrab, a.C);
         for (int I = I0; I < Iend; ++I) {
             const int s0 = a.cell_off[I], nI = a.cell_off[I + 1] - s0;
@@ -1473,9 +1487,9 @@ __global__ void __launch_bounds__(kPairThreads) pair_bwd64(BwdArgs b) {
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) gather_grad(const int *order, int64_t nb, const T *g, void *vs, int f64) {
+__global__ void __launch_bounds__(256) gather_grad(const int *order, const int *nb, const T *g, void *vs, int f64) {
     int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nb) return;
+    if (s >= *nb) return;
     int k = order[s];
     if (f64) {
         double *v = (double *)vs + 4 * (size_t)s;
@@ -1487,7 +1501,7 @@ __global__ void __launch_bounds__(256) gather_grad(const int *order, int64_t nb,
 }
 
 // Totals of the species-gradient slots over the stripe rows (one warp per slot).
-__global__ void __launch_bounds__(kGradSlots * 32) finish_bwd(const double *acc, int S, double *ge, double *gs) {
+__global__ void __launch_bounds__(kGradSlots * 32) finish_bwd(double *acc, int S, double *ge, double *gs) {
     const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double v = 0.0;
     for (int r = lane; r < kStripes; r += 32) v += acc[kAccStripes + r * kParts + i];
@@ -1500,6 +1514,7 @@ __global__ void __launch_bounds__(kGradSlots * 32) finish_bwd(const double *acc,
             gs[q] = v;
         }
     }
+    clear_sums(acc);
 }
 
 // ------------------------------------------------------ FP32 cluster kernel
@@ -1524,7 +1539,7 @@ __global__ void __launch_bounds__(kGradSlots * 32) finish_bwd(const double *acc,
 // multiples of 2^-q (xloc) plus a remainder (xlo), run shifts likewise, so
 // (x_k,hi - x_l,hi - shift_hi) is exact and adding the remainders rounds once.
 // Every force accumulator's .w sums |f|^2 over the molecule's pairs: the
-// scale of the FP32 error of its force (see flag_ill_conditioned and
+// scale of the FP32 error of its force (see finish_forces and
 // refine_ds).
 constexpr int kCT = 128, kCW = kCT / 32;
 // A molecule's FP32 force error is about a multiple of sqrt(sum_l |f_kl|^2)
@@ -1703,6 +1718,7 @@ __global__ void __launch_bounds__(kCT, MINB) pair_fwd32c(PairArgs a, ClKArgs c) 
     __shared__ float4 tab[kMaxSpecies * kMaxSpecies];
     __shared__ double dsums[kCW][8];
     for (int i = threadIdx.x; i < kMaxSpecies * kMaxSpecies; i += blockDim.x) tab[i] = a.tab.f[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && a.zero_word) *a.zero_word = 0;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     WarpC &w = wsh[wib];
     if (lane < 8) dsums[wib][lane] = 0.0;
@@ -2086,15 +2102,41 @@ ClKArgs cluster_args(aica_mesh *m) {
     return c;
 }
 
+// Waits for the call and reports the error bits of the last binning (the force
+// kernels set none).
 aica_status check_flags(aica_mesh *m, cudaStream_t st) {
     unsigned flags = 0;
-    AICA_CUDA(cudaMemcpyAsync(&flags, m->flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
-    AICA_CUDA(cudaStreamSynchronize(st));
+    if (m->pub_valid) {
+        AICA_CUDA(cudaStreamSynchronize(st));
+        flags = m->pub_flags;
+    } else {
+        AICA_CUDA(cudaMemcpyAsync(&flags, m->flags.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+        AICA_CUDA(cudaStreamSynchronize(st));
+    }
     if (flags & kFlagSpecies) { set_error("species index out of range"); return AICA_ERR_INVALID_ARG; }
     if (flags & kFlagOutside) { set_error("some molecules lie in no cell"); return AICA_ERR_OUTSIDE_MESH; }
     if (flags & kFlagCapacity) { set_error("a kernel capacity was exceeded"); return AICA_ERR_CAPACITY; }
     return AICA_OK;
 }
+
+// Accumulators and sums are zero when a call starts: its last kernel left them
+// so (two memsets per call less; with those of the binning and its copies a step
+// of 2 048 molecules goes from 18 stream operations to 10, 120 -> 94 us, checked
+// forces of 4 000 from 188 to 157 us), or they are cleared here (first call, new buffers, after a failed call).
+// settle() is for the end of the call's launches.
+struct CleanStart {
+    aica_mesh *m;
+    cudaStream_t st;
+    bool was;
+    aica_status begin() {
+        was = m->facc_clean && m->acc_clean;
+        if (!m->facc_clean && m->facc.p) AICA_CUDA(cudaMemsetAsync(m->facc.p, 0, m->facc.bytes, st));
+        if (!m->acc_clean) AICA_CUDA(cudaMemsetAsync(m->acc.p, 0, (kAccStripes + kStripes * kParts) * sizeof(double), st));
+        m->facc_clean = m->acc_clean = false;
+        return AICA_OK;
+    }
+    void settle() { m->facc_clean = m->acc_clean = was || really_ran(st); }
+};
 
 template <bool XF>
 void launch_fwd64(const PairArgs &a, bool multi, bool shift, int grid, cudaStream_t st) {
@@ -2231,11 +2273,7 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
     m->launches = 0;
     const int64_t n = m->n_mol;
     const bool f64 = prec == AICA_FP64;
-    if (n > 0) AICA_CUDA(cudaMemsetAsync(m->facc.p, 0, (f64 ? 4 * sizeof(double) : sizeof(float4)) * n, st));
-    AICA_CUDA(cudaMemsetAsync(m->acc.p, 0, (kAccStripes + kStripes * kParts) * sizeof(double), st));
     const bool multi = a.S > 1, shift = lj->shift != 0;
-    cudaEvent_t tstop;
-    AICA_CUDA(timing_begin(m, st, &tstop));
     // FP32 with box periodicity: the cluster kernel when the lists have a
     // cluster schedule (the cell kernel on request, and for general transforms)
     const bool clsched = !a.xf && m->n_cl_runs >= 0;
@@ -2248,6 +2286,18 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
         set_error("aica_forces: portion mode (halo molecules) needs box periodicity");
         return AICA_ERR_INVALID_ARG;
     }
+    // FP32 cluster path: molecules whose FP32 force cannot
+    // be certified to the tolerance are recomputed in double-single arithmetic
+    // (needs the cluster lists)
+    const bool refine = clpath && m->refine_tol > 0 && n > 0;
+    int *flags = refine ? m->flag_list.as<int>() : nullptr;
+    const float kf = refine ? (float)(kRefineScale / m->refine_tol) : 0.f;
+    a.zero_word = flags;                  // the flag count, for finish_forces
+    CleanStart clean{m, st, false};
+    s = clean.begin();
+    if (s != AICA_OK) return s;
+    cudaEvent_t tstop;
+    AICA_CUDA(timing_begin(m, st, &tstop));
     const ClKArgs c = cluster_args(m);
     bool cl64 = false;                 // FP64 cluster kernel
     if (!f64) {
@@ -2273,22 +2323,11 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
             a.cell_off, a.run_off, a.runs, a.C, acc);
         m->launches += 1;
     }
-    // FP32 cluster path: molecules whose FP32 force cannot
-    // be certified to the tolerance are recomputed in double-single arithmetic
-    // (needs the cluster lists)
-    const bool refine = clpath && m->refine_tol > 0 && n > 0;
-    int *flags = refine ? m->flag_list.as<int>() : nullptr;
-    if (refine) AICA_CUDA(cudaMemsetAsync(flags, 0, sizeof(int), st));
-    const float kf = refine ? (float)(kRefineScale / m->refine_tol) : 0.f;
     if (n > 0) {
         const unsigned g = (unsigned)((n + 255) / 256);
-        if (f64) unsort_forces<double><<<g, 256, 0, st>>>(m->inv.as<int>(), n, m->facc.p, (double *)force_out, 1, acc, ev_out, (long long *)counts_out);
-        else unsort_forces<float><<<g, 256, 0, st>>>(m->inv.as<int>(), n, m->facc.p, (float *)force_out, 0, acc, ev_out, (long long *)counts_out);
-        if (refine) {
-            flag_ill_conditioned<<<g, 256, 0, st>>>((const float4 *)m->facc.p, m->xloc.as<float4>(), (int)n, kf * kf,
-                                                    flags);
-            m->launches += 1;
-        }
+        const int *off = m->cell_off.as<int>(), *ord = m->order.as<int>(), *inv = m->inv.as<int>();
+        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, a.C, ord, inv, n, m->facc.p, (double *)force_out, acc, ev_out, (long long *)counts_out, nullptr, 0.f, nullptr);
+        else finish_forces<float><<<g, 256, 0, st>>>(off, a.C, ord, inv, n, m->facc.p, (float *)force_out, acc, ev_out, (long long *)counts_out, m->xloc.as<float4>(), refine ? kf * kf : 0.f, flags);
     } else {
         finish_sums<<<1, 15 * 32, 0, st>>>(acc, ev_out, (long long *)counts_out);
     }
@@ -2323,11 +2362,12 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
         }
         r.rc2h = (float)a.rc2_d;
         r.rc2l = (float)(a.rc2_d - (double)r.rc2h);
-        r.next = (unsigned *)(m->acc.as<double>() + 25);      // zeroed with the sums at the call's start
+        r.next = (unsigned *)(m->acc.as<double>() + 25);      // cleared by finish_forces
         refine_ds<<<152 * 8, 256, 0, st>>>(a, r);
         m->launches += 1;
     }
     AICA_CUDA(cudaGetLastError());
+    clean.settle();
     if (!m->deferred) return check_flags(m, st);
     return AICA_OK;
 }
@@ -2369,20 +2409,17 @@ extern "C" aica_status aica_forces_backward(aica_mesh *m, const aica_lj *lj, aic
     m->launches = 0;
     const int64_t n = m->n_mol;
     const bool f64 = prec == AICA_FP64, multi = b.S > 1;
-    const size_t esz = f64 ? 4 * sizeof(double) : sizeof(float4);
-    int nb = 0;
-    AICA_CUDA(cudaMemcpyAsync(&nb, m->cell_off.as<int>() + m->n_cells, sizeof(int), cudaMemcpyDeviceToHost, st));
-    AICA_CUDA(cudaStreamSynchronize(st));
     int launches = 0;
+    CleanStart clean{m, st, false};
+    s = clean.begin();
+    if (s != AICA_OK) return s;
+    const unsigned g = (unsigned)((n + 255) / 256);
+    const int *off = m->cell_off.as<int>(), *ord = m->order.as<int>(), *inv = m->inv.as<int>();
     if (n > 0) {
-        AICA_CUDA(cudaMemsetAsync(m->facc.p, 0, esz * n, st));
-        if (nb > 0) {
-            if (f64) gather_grad<double><<<(nb + 255) / 256, 256, 0, st>>>(m->order.as<int>(), nb, (const double *)grad_force, m->vsorted.p, 1);
-            else gather_grad<float><<<(nb + 255) / 256, 256, 0, st>>>(m->order.as<int>(), nb, (const float *)grad_force, m->vsorted.p, 0);
-            launches++;
-        }
+        if (f64) gather_grad<double><<<g, 256, 0, st>>>(ord, off + m->n_cells, (const double *)grad_force, m->vsorted.p, 1);
+        else gather_grad<float><<<g, 256, 0, st>>>(ord, off + m->n_cells, (const float *)grad_force, m->vsorted.p, 0);
+        launches++;
     }
-    AICA_CUDA(cudaMemsetAsync(m->acc.p, 0, (kAccStripes + kStripes * kParts) * sizeof(double), st));
     b.p.vs = m->vsorted.p;
     cudaEvent_t tstop;
     AICA_CUDA(timing_begin(m, st, &tstop));
@@ -2396,16 +2433,15 @@ extern "C" aica_status aica_forces_backward(aica_mesh *m, const aica_lj *lj, aic
     AICA_CUDA(timing_end(tstop, st));
     launches++;
     if (n > 0) {
-        if (f64) unsort_forces<double><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m->inv.as<int>(), n, m->facc.p, (double *)grad_pos, 1);
-        else unsort_forces<float><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m->inv.as<int>(), n, m->facc.p, (float *)grad_pos, 0);
+        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, b.p.C, ord, inv, n, m->facc.p, (double *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr);
+        else finish_forces<float><<<g, 256, 0, st>>>(off, b.p.C, ord, inv, n, m->facc.p, (float *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr);
         launches++;
     }
-    if (grad_eps || grad_sigma) {
-        finish_bwd<<<1, kGradSlots * 32, 0, st>>>(m->acc.as<double>(), b.S, grad_eps, grad_sigma);
-        launches++;
-    }
+    finish_bwd<<<1, kGradSlots * 32, 0, st>>>(m->acc.as<double>(), b.S, grad_eps, grad_sigma);
+    launches++;
     m->launches = launches;
     AICA_CUDA(cudaGetLastError());
+    clean.settle();
     if (!m->deferred) return check_flags(m, st);
     return AICA_OK;
 }

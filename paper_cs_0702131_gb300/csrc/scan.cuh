@@ -123,7 +123,7 @@ static __device__ __forceinline__ unsigned long long scan_word(unsigned epoch, u
 
 static __global__ void __launch_bounds__(kScanThreads) scan_lookback(const int *in, int64_t n, int *out,
                                                               unsigned long long *state, unsigned *flags,
-                                                              unsigned timeout_flag) {
+                                                              unsigned timeout_flag, int *zero) {
     __shared__ int sh[kScanThreads / 32];
     __shared__ unsigned s_tile, s_epoch;
     __shared__ int s_prefix;
@@ -193,6 +193,7 @@ static __global__ void __launch_bounds__(kScanThreads) scan_lookback(const int *
         if (lane == 0) {
             s_prefix = prefix;
             if (tile == gridDim.x - 1) {
+                if (zero) *zero = 0;
                 ((volatile unsigned long long *)state)[0] = 0ull;
                 ((volatile unsigned long long *)state)[1] = (unsigned long long)((epoch + 1u) & 0x3fffffffu);
             }
@@ -210,11 +211,12 @@ static __global__ void __launch_bounds__(kScanThreads) scan_lookback(const int *
 // Words of state that scan_lookback needs for n values.
 inline int64_t scan_lookback_words(int64_t n) { return 2 + (n + 1 + kScanTile - 1) / kScanTile; }
 
-// Exclusive scan of n int values into out[0..n] in one launch.
+// Exclusive scan of n int values into out[0..n] in one launch; zero (optional):
+// a word of an earlier kernel to clear on the way.
 inline int exclusive_scan_1pass(const int *in, int64_t n, int *out, unsigned long long *state, unsigned *flags,
-                                unsigned timeout_flag, cudaStream_t st) {
+                                unsigned timeout_flag, int *zero, cudaStream_t st) {
     const int64_t tiles = (n + 1 + kScanTile - 1) / kScanTile;
-    scan_lookback<<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, out, state, flags, timeout_flag);
+    scan_lookback<<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, out, state, flags, timeout_flag, zero);
     return 1;
 }
 
