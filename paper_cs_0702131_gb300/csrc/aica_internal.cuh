@@ -226,7 +226,7 @@ struct aica_mesh {
     // force accumulators, the sums, the species word of the flags.  False until
     // cleared, and again from the start of a call until its launches succeeded.
     bool bin_clean = false, facc_clean = false, acc_clean = false, flags_clean = false;
-    // Flags of the last checked binning, written by its last block to mapped
+    // Flags of the last checked binning, written by publish_flags to mapped
     // host memory (pub; NULL if there is none).
     unsigned *pub = nullptr, *pub_dev = nullptr;
     bool pub_valid = false;                  // pub_flags are the device's error bits

@@ -79,8 +79,7 @@ struct BinArgs {
     int *cell_of;
     int *cnt;              // molecules per cell (counted as they are located)
     int *inv;              // original -> binned index; -1 for molecules in no cell
-    unsigned *flags;       // [0] error bits, [1] largest species index, [2] blocks that are done
-    unsigned *pub;         // host: flags[0], flags[1] of this call (checked calls; NULL: not written)
+    unsigned *flags;       // [0] error bits, [1] largest species index
 };
 
 // Add one molecule to cell c's count (c < 0: none), aggregated over the warp's
@@ -592,21 +591,6 @@ __device__ __forceinline__ void frame_split(const BinArgs &a, const double *p, c
 // coordinates local to the cell's molecule-frame origin into binned order, record the
 // inverse permutation, and the cell's bounding sphere (centre = mean, radius
 // = largest distance, rounded up) that the pair kernels cull with.
-// End of a binning's last kernel: its last block hands the flags to the host
-// (instead of a copy after it) and leaves the species word zero.
-__device__ __forceinline__ void publish_flags(const BinArgs &a) {
-    if (!a.pub) return;
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    __threadfence();
-    if (atomicAdd(a.flags + 2, 1u) != gridDim.x - 1) return;
-    __threadfence();
-    a.pub[0] = atomicAdd(a.flags, 0u);
-    a.pub[1] = atomicExch(a.flags + 1, 0u);
-    a.flags[2] = 0;
-    __threadfence_system();
-}
-
 template <int G>
 __global__ void __launch_bounds__(256) bin_cells(BinArgs a, const int *cell_off, int C, int *order, double *xs64,
                                                  float4 *xloc, float4 *sph) {
@@ -706,7 +690,6 @@ __global__ void __launch_bounds__(256) bin_cells(BinArgs a, const int *cell_off,
     const int mx = __reduce_max_sync(0xffffffffu, spmax);
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.flags, kFlagSpecies);
     if (lane == 0 && mx > 0) atomicMax((int *)a.flags + 1, mx);
-    publish_flags(a);
 }
 
 // The same per slot, for cells of a few molecules.  Warp w owns the cells
@@ -761,8 +744,9 @@ __device__ __forceinline__ float4 sphere_of(const float4 *x, int m) {
     return make_float4(cx, cy, cz, sqrtf(rr) * (1.f + 1e-5f) + 1e-5f);
 }
 
-__device__ __forceinline__ void bin_slots_warp(const BinArgs &a, const int *cell_off, const int *nbp, const int *un,
-                                               const int *ucell, int *order, double *xs64, float4 *xloc, float4 *sph) {
+__global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const int *cell_off, const int *nbp,
+                                                             const int *un, const int *ucell, int *order,
+                                                             double *xs64, float4 *xloc, float4 *sph) {
     __shared__ int sk[kSlotWarps][64];
     __shared__ float4 sx[kSlotWarps][64];
     const unsigned FULL = 0xffffffffu;
@@ -860,11 +844,15 @@ __device__ __forceinline__ void bin_slots_warp(const BinArgs &a, const int *cell
     if (lane == 0 && mx > 0) atomicMax((int *)a.flags + 1, mx);
 }
 
-__global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const int *cell_off, const int *nbp,
-                                                             const int *un, const int *ucell, int *order,
-                                                             double *xs64, float4 *xloc, float4 *sph) {
-    bin_slots_warp(a, cell_off, nbp, un, ucell, order, xs64, xloc, sph);
-    publish_flags(a);
+// Hands the flags of a checked binning to the host (mapped memory) and leaves
+// the flag words zero unless an error was found.  A launch of its own: counting
+// the blocks in the last kernel needs a fence per block, which made it 63 -> 86
+// us for 1 030 000 molecules (18 -> 25 for 256 000); a copy and a memset cost more.
+__global__ void publish_flags(unsigned *flags, unsigned *pub) {
+    pub[0] = flags[0];
+    pub[1] = flags[1];
+    flags[1] = 0;
+    __threadfence_system();
 }
 
 }  // namespace
@@ -966,9 +954,8 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     a.cnt = cnt;
     a.inv = m->inv.as<int>();
     // with deferred checks the error bits (flags[0]) accumulate until
-    // aica_check_status; a checked call's last kernel hands them to the host
+    // aica_check_status; a checked call hands them to the host at its end
     const bool publish = !m->deferred && m->pub && n > 0 && C > 0;
-    a.pub = publish ? m->pub_dev : nullptr;
     if (!m->deferred && !m->flags_clean) AICA_CUDA(cudaMemsetAsync(m->flags.p, 0, 16, st));
     m->flags_clean = m->pub_valid = false;
     const bool was_clean = m->bin_clean;
@@ -1022,7 +1009,11 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->max_species = -1;
     if (!m->deferred) {
         unsigned flags[2] = {0, 0};
-        if (!publish) AICA_CUDA(cudaMemcpyAsync(flags, m->flags.p, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+        if (publish) {
+            publish_flags<<<1, 1, 0, st>>>(m->flags.as<unsigned>(), m->pub_dev);
+            AICA_CUDA(cudaGetLastError());
+            m->launches += 1;
+        } else AICA_CUDA(cudaMemcpyAsync(flags, m->flags.p, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
         AICA_CUDA(cudaStreamSynchronize(st));
         if (publish) {
             flags[0] = ((volatile unsigned *)m->pub)[0];

@@ -106,12 +106,12 @@ __device__ __forceinline__ void finish_value(double *acc, double *ev, long long 
     }
 }
 
-// Leave the sums' rows and the unit counters zero for the next call (a whole
+// Leave the sums' rows and the unit counter zero for the next call (a whole
 // block, after its finish_value calls).
 __device__ __forceinline__ void clear_sums(double *acc) {
     __syncthreads();
     for (int i = threadIdx.x; i < kStripes * kParts; i += blockDim.x) acc[kAccStripes + i] = 0.0;
-    if (threadIdx.x < 2) acc[24 + threadIdx.x] = 0.0;
+    if (threadIdx.x == 0) acc[24] = 0.0;
 }
 
 // One warp per value (15 warps); used when no molecule was binned (otherwise
@@ -791,21 +791,22 @@ __global__ void __launch_bounds__(kPairThreads) pair_fwd64(PairArgs a) {
 }
 
 // ---------------------------------------------------------------- results
-// One pass over the binned molecules (cell_off[C] of them): forces to the
-// original order (rows of molecules in no cell are zero), the totals of the
-// pair kernel's striped sums (acc, in the first block), and the flag list
-// (kflag2 > 0): the FP32 error of a molecule's force is about a fixed multiple of
+// One pass over the molecules: forces to the original order (rows of molecules
+// in no cell are zero), the totals of the pair kernel's striped sums (acc, in
+// the first block; left zero for the next call), and the flag list (kflag2 > 0):
+// the FP32 error of a molecule's force is about a fixed multiple of
 // sqrt(sum |f|^2) (the .w of its accumulator); a molecule whose force is too
 // small against it goes to the list for recomputation.  The list follows the
-// binned order (one append per block), so the molecules' positions.
-// Accumulators and sums are left zero for the next call.  Memory-bound and
-// small, so what counts is the launches: this one takes the place of two
-// kernels (256 000 molecules: 6.1 and 4.9 us) and of two memsets per call.
+// binned order (one append per block), so the molecules' positions.  Thread k
+// gathers the row of molecule k and tests the accumulator k, so both the writes
+// of 12 bytes a row and the test are in order: scattering each row to its
+// molecule instead took 91 us for 1 030 000 molecules (the two passes that this
+// one replaces: 11.4 and 11.4).
 template <class T>
-__global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C, const int *order, const int *inv,
-                                                     int64_t n, void *facc, T *out, double *acc, double *ev,
+__global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C, const int *inv, int64_t n,
+                                                     const void *facc, T *out, double *acc, double *ev,
                                                      long long *counts, const float4 *xloc, float kflag2,
-                                                     int *flag_list) {
+                                                     int *flag_list, int *flag_count) {
     __shared__ int wcnt[8], wbase[8];
     if (acc && blockIdx.x == 0) {
         for (int i = threadIdx.x >> 5; i < 15; i += blockDim.x >> 5) finish_value(acc, ev, counts, i, threadIdx.x & 31);
@@ -813,25 +814,29 @@ __global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C,
     }
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool f = false;
-    if (k < n && inv[k] < 0) out[3 * k] = out[3 * k + 1] = out[3 * k + 2] = (T)0;
-    if (k < cell_off[C]) {
-        T *o = out + 3 * (int64_t)order[k];
-        if (sizeof(T) == 8) {
-            double2 *v = (double2 *)facc + 2 * k;
-            const double2 xy = v[0];
-            const double z = v[1].x;
-            v[0] = v[1] = make_double2(0.0, 0.0);
-            o[0] = (T)xy.x;
-            o[1] = (T)xy.y;
-            o[2] = (T)z;
-        } else {
-            const float4 v = ((float4 *)facc)[k];
-            ((float4 *)facc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            o[0] = (T)v.x;
-            o[1] = (T)v.y;
-            o[2] = (T)v.z;
-            f = kflag2 > 0.f && v.x * v.x + v.y * v.y + v.z * v.z < kflag2 * v.w &&
-                !(__float_as_int(xloc[k].w) & kGhostBit);
+    if (k < n) {
+        const int s = inv[k];
+        T x = 0, y = 0, z = 0;
+        if (s >= 0) {
+            if (sizeof(T) == 8) {
+                const double2 *v = (const double2 *)facc + 2 * (size_t)s;
+                const double2 xy = v[0];
+                x = (T)xy.x;
+                y = (T)xy.y;
+                z = (T)v[1].x;
+            } else {
+                const float4 v = ((const float4 *)facc)[s];
+                x = (T)v.x;
+                y = (T)v.y;
+                z = (T)v.z;
+            }
+        }
+        out[3 * k] = x;
+        out[3 * k + 1] = y;
+        out[3 * k + 2] = z;
+        if (kflag2 > 0.f && k < cell_off[C]) {
+            const float4 v = ((const float4 *)facc)[k];
+            f = v.x * v.x + v.y * v.y + v.z * v.z < kflag2 * v.w && !(__float_as_int(xloc[k].w) & kGhostBit);
         }
     }
     if (!(kflag2 > 0.f)) return;
@@ -845,7 +850,7 @@ __global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C,
             wbase[i] = t;
             t += wcnt[i];
         }
-        const int base = t ? atomicAdd(flag_list, t) : 0;
+        const int base = t ? atomicAdd(flag_count, t) : 0;
         for (int i = 0; i < 8; ++i) wbase[i] += base;
     }
     __syncthreads();
@@ -898,7 +903,8 @@ __device__ __forceinline__ ds ds_rcp(ds a) {
 // operation order decides, so the pair set is exactly the pairs within rc.
 // Writes the force (original order) over the FP32 one.
 struct RefineArgs {
-    const int *flag_list, *cl_first, *cl_of, *full_off, *order;
+    int *flag_list;              // [0] count (written at the end), [1..] flagged molecules
+    const int *cl_first, *cl_of, *full_off, *order;
     const unsigned long long *full;
     const float4 *xlo;
     const float4 *cl_box;        // boxes of the clusters' molecules from the FP32 pass
@@ -910,7 +916,11 @@ struct RefineArgs {
     float sig2[kMaxSpecies * kMaxSpecies][2];   // sigma_ab^2 and 24 eps_ab, double-single
     float c24[kMaxSpecies * kMaxSpecies][2];
     float rc2h, rc2l;            // rc^2, double-single
-    unsigned *next;              // next unclaimed entry of the flag list (zero at launch)
+    unsigned *next;              // next unclaimed entry of the flag list
+    unsigned *done;              // blocks that are done
+    int *count;                  // entries of the flag list; all three are left zero
+    float4 *facc;                // force accumulators (read by now), cleared for the next call
+    int64_t n;                   // their number
 };
 
 constexpr int kRefineGrab = 4;        // flagged molecules claimed per warp at a time
@@ -922,7 +932,9 @@ __global__ void __launch_bounds__(256) refine_ds(PairArgs a, RefineArgs r) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u, le = FULL >> (31 - lane);
-    const int nflag = r.flag_list[0];
+    const int nflag = *r.count;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < r.n; i += (int64_t)gridDim.x * blockDim.x)
+        r.facc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     const float pre2 = a.rc2_hi * 1.001f + 1e-3f;
     const float reach = sqrtf(pre2) + 1e-3f;
     // warps claim consecutive entries of the (spatially ordered) list, up to
@@ -1117,6 +1129,14 @@ __global__ void __launch_bounds__(256) refine_ds(PairArgs a, RefineArgs r) {
             r.out[3 * (size_t)o + 2] = Fz.h + Fz.l;
         }
     }
+    }
+    // the last block to get here leaves the counters zero: every block has read them
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(r.done, 1u) == gridDim.x - 1) {
+        r.flag_list[0] = nflag;
+        *r.count = 0;
+        *r.next = 0;
+        *r.done = 0;
     }
 }
 
@@ -1718,7 +1738,6 @@ __global__ void __launch_bounds__(kCT, MINB) pair_fwd32c(PairArgs a, ClKArgs c) 
     __shared__ float4 tab[kMaxSpecies * kMaxSpecies];
     __shared__ double dsums[kCW][8];
     for (int i = threadIdx.x; i < kMaxSpecies * kMaxSpecies; i += blockDim.x) tab[i] = a.tab.f[i];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.zero_word) *a.zero_word = 0;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     WarpC &w = wsh[wib];
     if (lane < 8) dsums[wib][lane] = 0.0;
@@ -2119,10 +2138,8 @@ aica_status check_flags(aica_mesh *m, cudaStream_t st) {
     return AICA_OK;
 }
 
-// Accumulators and sums are zero when a call starts: its last kernel left them
-// so (two memsets per call less; with those of the binning and its copies a step
-// of 2 048 molecules goes from 18 stream operations to 10, 120 -> 94 us, checked
-// forces of 4 000 from 188 to 157 us), or they are cleared here (first call, new buffers, after a failed call).
+// Accumulators and sums are zero when a call starts: the one before left them
+// so, or they are cleared here (first call, new buffers, after a failed call).
 // settle() is for the end of the call's launches.
 struct CleanStart {
     aica_mesh *m;
@@ -2292,7 +2309,6 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
     const bool refine = clpath && m->refine_tol > 0 && n > 0;
     int *flags = refine ? m->flag_list.as<int>() : nullptr;
     const float kf = refine ? (float)(kRefineScale / m->refine_tol) : 0.f;
-    a.zero_word = flags;                  // the flag count, for finish_forces
     CleanStart clean{m, st, false};
     s = clean.begin();
     if (s != AICA_OK) return s;
@@ -2325,9 +2341,9 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
     }
     if (n > 0) {
         const unsigned g = (unsigned)((n + 255) / 256);
-        const int *off = m->cell_off.as<int>(), *ord = m->order.as<int>(), *inv = m->inv.as<int>();
-        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, a.C, ord, inv, n, m->facc.p, (double *)force_out, acc, ev_out, (long long *)counts_out, nullptr, 0.f, nullptr);
-        else finish_forces<float><<<g, 256, 0, st>>>(off, a.C, ord, inv, n, m->facc.p, (float *)force_out, acc, ev_out, (long long *)counts_out, m->xloc.as<float4>(), refine ? kf * kf : 0.f, flags);
+        const int *off = m->cell_off.as<int>(), *inv = m->inv.as<int>();
+        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, a.C, inv, n, m->facc.p, (double *)force_out, acc, ev_out, (long long *)counts_out, nullptr, 0.f, nullptr, nullptr);
+        else finish_forces<float><<<g, 256, 0, st>>>(off, a.C, inv, n, m->facc.p, (float *)force_out, acc, ev_out, (long long *)counts_out, m->xloc.as<float4>(), refine ? kf * kf : 0.f, flags, (int *)(acc + 27));
     } else {
         finish_sums<<<1, 15 * 32, 0, st>>>(acc, ev_out, (long long *)counts_out);
     }
@@ -2362,9 +2378,15 @@ extern "C" aica_status aica_forces(aica_mesh *m, const aica_lj *lj, aica_precisi
         }
         r.rc2h = (float)a.rc2_d;
         r.rc2l = (float)(a.rc2_d - (double)r.rc2h);
-        r.next = (unsigned *)(m->acc.as<double>() + 25);      // cleared by finish_forces
+        r.next = (unsigned *)(acc + 25);
+        r.done = (unsigned *)(acc + 26);
+        r.count = (int *)(acc + 27);
+        r.facc = m->facc.as<float4>();
+        r.n = n;
         refine_ds<<<152 * 8, 256, 0, st>>>(a, r);
         m->launches += 1;
+    } else if (n > 0) {
+        AICA_CUDA(cudaMemsetAsync(m->facc.p, 0, (f64 ? 4 * sizeof(double) : sizeof(float4)) * n, st));
     }
     AICA_CUDA(cudaGetLastError());
     clean.settle();
@@ -2433,10 +2455,11 @@ extern "C" aica_status aica_forces_backward(aica_mesh *m, const aica_lj *lj, aic
     AICA_CUDA(timing_end(tstop, st));
     launches++;
     if (n > 0) {
-        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, b.p.C, ord, inv, n, m->facc.p, (double *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr);
-        else finish_forces<float><<<g, 256, 0, st>>>(off, b.p.C, ord, inv, n, m->facc.p, (float *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr);
+        if (f64) finish_forces<double><<<g, 256, 0, st>>>(off, b.p.C, inv, n, m->facc.p, (double *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr, nullptr);
+        else finish_forces<float><<<g, 256, 0, st>>>(off, b.p.C, inv, n, m->facc.p, (float *)grad_pos, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr, nullptr);
         launches++;
     }
+    if (n > 0) AICA_CUDA(cudaMemsetAsync(m->facc.p, 0, (f64 ? 4 * sizeof(double) : sizeof(float4)) * n, st));
     finish_bwd<<<1, kGradSlots * 32, 0, st>>>(m->acc.as<double>(), b.S, grad_eps, grad_sigma);
     launches++;
     m->launches = launches;

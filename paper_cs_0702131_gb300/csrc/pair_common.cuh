@@ -35,7 +35,6 @@ struct PairArgs {
     const void *vs;              // backward: grad_force in binned order (float4 / double4)
     double *acc;                 // [0..6] U, W; [8..15] counters (as unsigned long long); [16..] grads
     unsigned *next_cell;         // FP32 kernel: next unclaimed cell (zero at launch)
-    int *zero_word;              // FP32 cluster kernel: a word to clear for a later kernel (NULL: none)
     int ghosts;                  // portion mode: xloc.w carries kGhostBit on halo molecules
     int xf;                      // general referring transforms: image field = transform index
     int n_xf;                    // transforms in xft
