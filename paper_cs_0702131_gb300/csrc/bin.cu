@@ -844,10 +844,11 @@ __global__ void __launch_bounds__(kSlotWarps * 32) bin_slots(BinArgs a, const in
     if (lane == 0 && mx > 0) atomicMax((int *)a.flags + 1, mx);
 }
 
-// Hands the flags of a checked binning to the host (mapped memory) and leaves
-// the flag words zero unless an error was found.  A launch of its own: counting
-// the blocks in the last kernel needs a fence per block, which made it 63 -> 86
-// us for 1 030 000 molecules (18 -> 25 for 256 000); a copy and a memset cost more.
+// Hands the flags of a checked binning to the host (mapped memory, in place of
+// a copy and of a memset before the next call) and leaves the species word
+// zero.  A launch of its own: counting the blocks in the last kernel needs a
+// fence per block, which made it 63 -> 86 us for 1 372 000 molecules (18 -> 25
+// for 256 000).
 __global__ void publish_flags(unsigned *flags, unsigned *pub) {
     pub[0] = flags[0];
     pub[1] = flags[1];

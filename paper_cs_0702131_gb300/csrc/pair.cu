@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(kPairThreads) pair_fwd64(PairArgs a) {
 // binned order (one append per block), so the molecules' positions.  Thread k
 // gathers the row of molecule k and tests the accumulator k, so both the writes
 // of 12 bytes a row and the test are in order: scattering each row to its
-// molecule instead took 91 us for 1 030 000 molecules (the two passes that this
+// molecule instead took 91 us for 1 372 000 molecules (the two passes that this
 // one replaces: 11.4 and 11.4).
 template <class T>
 __global__ void __launch_bounds__(256) finish_forces(const int *cell_off, int C, const int *inv, int64_t n,
@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(256) refine_ds(PairArgs a, RefineArgs r) {
         const int k = r.flag_list[1 + i];
         // k's cell stands in its remainder's .w, each cluster's molecule range beside
         // its box: fewer dependent loads per molecule than a search of cell_off and
-        // the offsets by cell (cut-off 3, 1 030 000 molecules, whole step: 1387 ->
+        // the offsets by cell (cut-off 3, 1 372 000 molecules, whole step: 1387 ->
         // 1377 us; channel of a million 1057 -> 1048)
         const float4 xlk = r.xlo[k];
         const int A = r.cl_of[__float_as_int(xlk.w)];
@@ -1295,11 +1295,13 @@ __global__ void __launch_bounds__(kThreads32, MINB) pair_bwd32(BwdArgs b) {
     int ncell = 0;
     // the first cells by warp, the next ones claimed while these are worked on:
     // with enough warps for all cells the grouping of the species' FP32 sums, so
-    // their last bits, does not depend on the order in which warps start
-    const int nwarps = gridDim.x * kWarps32;
-    int I0 = (blockIdx.x * kWarps32 + wib) * kGrab;
+    // their last bits, does not depend on the order in which warps start.  From
+    // lane 0, so that the compiler knows I0 for the same in all lanes: computed by
+    // each lane it cost 48 to 132 bytes of spills (8 388 608 molecules: 8.18 ->
+    // 8.78 ms)
+    int I0 = __shfl_sync(FULL, (blockIdx.x * kWarps32 + wib) * kGrab, 0);
     while (I0 < a.C) {
-        const int Inext = nwarps * kGrab + (lane == 0 ? (int)atomicAdd(a.next_cell, (unsigned)kGrab) : 0);
+        const int Inext = lane == 0 ? (int)(gridDim.x * (kWarps32 * kGrab) + atomicAdd(a.next_cell, (unsigned)kGrab)) : 0;
         const int Iend = min(I0 + kGrab, a.C);
         for (int I = I0; I < Iend; ++I) {
             const int s0 = a.cell_off[I], nI = a.cell_off[I + 1] - s0;
