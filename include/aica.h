@@ -329,7 +329,7 @@ aica_status aica_take_kernel_times(aica_mesh *mesh, float *ms, int64_t cap, int6
  *   AICA_OPT_COUNT_EVALUATED  (default 1) aica_forces fills counts_out[0..2]
  *       (pairs of every listed cell pair, §2.3) with an extra pass over the
  *       cell schedule when the FP32 cluster kernel runs; 0 skips that pass
- *       and reports 0 there.  The within-rc counts [3..5] are always exact.
+ *       and reports 0 there (FP64 forces always report them).  The within-rc counts [3..5] are always exact.
  *   AICA_OPT_FP32_KERNEL      (default 0) FP32 box-periodic pair kernel:
  *       0 the cluster kernel when the lists have a cluster schedule, 1 the
  *       cell kernel (for comparison; its forces are not refined).
