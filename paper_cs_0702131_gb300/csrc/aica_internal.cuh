@@ -117,8 +117,8 @@ __host__ __device__ inline int unpack_n(int32_t p, int axis) {
     return (int)(signed char)((p >> (8 * axis)) & 0xff);
 }
 
-// Whether words cleared by this call's own memset may count as clean for later
-// calls: not when the memset was only captured into a graph.
+// Whether the call's launches run now; not when they are only captured into a
+// graph (words cleared by its own memset then don't count as clean for later calls).
 inline bool really_ran(cudaStream_t st) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
@@ -231,6 +231,10 @@ struct aica_mesh {
     unsigned *pub = nullptr, *pub_dev = nullptr;
     bool pub_valid = false;                  // pub_flags are the device's error bits
     unsigned pub_flags = 0;
+    // A binning of this mesh was captured into a graph.  A replay changes the
+    // flag words without a host call, so from then on flags_clean and pub_flags
+    // say nothing: checked binnings clear the words, checked forces read them.
+    bool captured = false;
 
     bool deferred = false;
     int64_t launches = 0;

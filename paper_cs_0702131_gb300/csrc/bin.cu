@@ -871,6 +871,8 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int C = (int)m->n_cells;
+    const bool runs = really_ran(st);
+    if (!runs) m->captured = true;
     m->launches = 0;
     m->binned = false;
     if (n > m->cap_mol) {
@@ -957,7 +959,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     // with deferred checks the error bits (flags[0]) accumulate until
     // aica_check_status; a checked call hands them to the host at its end
     const bool publish = !m->deferred && m->pub && n > 0 && C > 0;
-    if (!m->deferred && !m->flags_clean) AICA_CUDA(cudaMemsetAsync(m->flags.p, 0, 16, st));
+    if (!m->deferred && (!m->flags_clean || m->captured)) AICA_CUDA(cudaMemsetAsync(m->flags.p, 0, 16, st));
     m->flags_clean = m->pub_valid = false;
     const bool was_clean = m->bin_clean;
     if (!was_clean) {
@@ -1002,7 +1004,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->n_mol_prev = n;
     m->hint_valid = true;
     AICA_CUDA(cudaGetLastError());
-    m->bin_clean = was_clean || really_ran(st);
+    m->bin_clean = was_clean || runs;
     if (cell_of && n) AICA_CUDA(cudaMemcpyAsync(cell_of, a.cell_of, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (order && n) AICA_CUDA(cudaMemcpyAsync(order, m->order.p, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (cell_off) AICA_CUDA(cudaMemcpyAsync(cell_off, off, sizeof(int) * (C + 1), cudaMemcpyDeviceToDevice, st));

@@ -2104,7 +2104,7 @@ ClKArgs cluster_args(aica_mesh *m) {
 // kernels set none).
 aica_status check_flags(aica_mesh *m, cudaStream_t st) {
     unsigned flags = 0;
-    if (m->pub_valid) {
+    if (m->pub_valid && !m->captured) {
         AICA_CUDA(cudaStreamSynchronize(st));
         flags = m->pub_flags;
     } else {
