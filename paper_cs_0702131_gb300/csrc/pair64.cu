@@ -363,7 +363,7 @@ bool fill_tab64(const PairArgs &a, const aica_lj *lj, Tab64 &T) {
 }  // namespace
 
 bool launch_fwd64c(const PairArgs &a, const ClKArgs &c, const aica_lj *lj, cudaStream_t st) {
-    Tab64 T;
+    Tab64 T{};       // zero where a species has no parameters: such pairs carry nothing
     if (!fill_tab64(a, lj, T)) return false;
     if (a.S > 1) {
         if (lj->shift) launch64c<true, true, false>(a, c, T, st);
@@ -376,7 +376,7 @@ bool launch_fwd64c(const PairArgs &a, const ClKArgs &c, const aica_lj *lj, cudaS
 }
 
 bool launch_bwd64c(const PairArgs &a, const ClKArgs &c, const aica_lj *lj, const BwdTab *t, cudaStream_t st) {
-    Tab64 T;
+    Tab64 T{};       // zero where a species has no parameters: such pairs carry nothing
     if (!fill_tab64(a, lj, T)) return false;
     for (int i = 0; i < a.S; ++i)
         for (int j = 0; j < a.S; ++j) {
