@@ -12,7 +12,11 @@
 // below 2^-62 before the last rounding); conversions are done on the bit
 // patterns, which would otherwise run on the FP64 pipe too; and the virial is
 // the sum of x (x) F over the forces a warp hands out (x in the cluster's
-// frame; each pair adds f and -f, so the origin cancels) instead of six products per pair.
+// frame; each pair adds f and -f, so the origin cancels) instead of six products
+// per pair.  A pair then carries an error of about 2^-53 |x| |f| where its virial is
+// r (x) f, so pairs much closer than their coordinates (r < rc / 8; none in a
+// fluid, some among overlapping molecules) hand out their force and
+// r (x) f directly.
 #include <algorithm>
 
 #include "cluster.cuh"
@@ -111,6 +115,7 @@ __global__ void __launch_bounds__(kW64 * 32) pair64c(PairArgs a, ClKArgs c, Tab6
     __syncthreads();
     const float pre2 = a.rc2_pre, rcut = sqrtf(pre2) * 1.00001f, rcut2 = rcut * rcut;
     const int rc_hi = __double2hiint(a.rc2_d);
+    const int close_hi = rc_hi - (6 << 20);              // r^2 below about rc^2 / 64
     double *facc = (double *)a.facc;
     const double *vs = (const double *)a.vs;
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -232,16 +237,23 @@ __global__ void __launch_bounds__(kW64 * 32) pair64c(PairArgs a, ClKArgs c, Tab6
                             } else {
                                 acc[0] = fma(i6, fma(P.C, i6, -P.D), acc[0]);
                                 if (SHIFT) acc[0] -= P.ush;
-                                fx = fma(-fs, rx, fx);
-                                fy = fma(-fs, ry, fy);
-                                fz = fma(-fs, rz, fz);
                             }
                             double *f = &w.col[0][t][lane & (kCols - 1)];
                             if (BWD) {
                                 f[0] += gx;
                                 f[kTile * kCols] += gy;
                                 f[2 * kTile * kCols] += gz;
+                            } else if (__double2hiint(r2) < close_hi) {
+                                gx = fs * rx;
+                                gy = fs * ry;
+                                gz = fs * rz;
+                                atomic_add3(facc + 4 * (size_t)(k0 + t), gx, gy, gz);
+                                atomic_add3(facc + 4 * (size_t)l, -gx, -gy, -gz);
+                                vir_add64(acc, rx, ry, rz, gx, gy, gz);
                             } else {
+                                fx = fma(-fs, rx, fx);
+                                fy = fma(-fs, ry, fy);
+                                fz = fma(-fs, rz, fz);
                                 f[0] = fma(fs, rx, f[0]);
                                 f[kTile * kCols] = fma(fs, ry, f[kTile * kCols]);
                                 f[2 * kTile * kCols] = fma(fs, rz, f[2 * kTile * kCols]);
