@@ -892,11 +892,12 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
         m->cap_mol = cap;
     }
     AICA_CUDA(m->cell_off.reserve(sizeof(int) * (C + 1)));
-    const void *old_fill = m->fill.p, *old_miss = m->miss.p;
+    // new memory is not clean, wherever it lies (a freed address may come again)
+    const size_t miss_bytes = sizeof(int) * (std::max<int64_t>(n, 1) + 1);
+    if (m->fill.bytes < sizeof(int) * (C + 1) || m->miss.bytes < miss_bytes) m->bin_clean = false;
     AICA_CUDA(m->fill.reserve(sizeof(int) * (C + 1)));
     AICA_CUDA(m->sph.reserve(sizeof(float4) * C));
-    AICA_CUDA(m->miss.reserve(sizeof(int) * (std::max<int64_t>(n, 1) + 1)));
-    if (m->fill.p != old_fill || m->miss.p != old_miss) m->bin_clean = false;
+    AICA_CUDA(m->miss.reserve(miss_bytes));
     m->n_mol = n;
     BinArgs a{};
     a.n = n;
