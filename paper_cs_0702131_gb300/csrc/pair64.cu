@@ -99,7 +99,9 @@ __device__ __forceinline__ void vir_add64(double (&v)[7], double x, double y, do
 // of slots.
 template <bool MULTI, bool SHIFT, bool BWD>
 __global__ void __launch_bounds__(kW64 * 32) pair64c(PairArgs a, ClKArgs c, Tab64 T, int parts) {
-    extern __shared__ double sh_raw[];
+    extern __shared__ __align__(16) unsigned char sh_raw[];
+    static_assert(alignof(Warp64<BWD>) == 16 && sizeof(Warp64<BWD>) % 16 == 0 && alignof(Slots64) <= 16,
+                  "the warps' shares are read with 16-byte loads");
     __shared__ Par64 tab[MULTI ? kMaxSpecies * kMaxSpecies : 1];
     if (MULTI)
         for (int i = threadIdx.x; i < kMaxSpecies * kMaxSpecies; i += blockDim.x) tab[i] = T.p[i];
