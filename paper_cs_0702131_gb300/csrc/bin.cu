@@ -80,6 +80,7 @@ struct BinArgs {
     int *cnt;              // molecules per cell (counted as they are located)
     int *inv;              // original -> binned index; -1 for molecules in no cell
     unsigned *flags;       // [0] error bits, [1] largest species index
+    int walkers;           // molecules of a warp that must have left their cells for them to walk
 };
 
 // Add one molecule to cell c's count (c < 0: none), aggregated over the warp's
@@ -119,78 +120,33 @@ __device__ __forceinline__ int orient(float3 a, float3 b, float3 c, float3 q, fl
     return s;
 }
 
-// q (p local to cell c) inside cell c with the SoS tie-break: 1 inside, 0
-// outside, -1 undecided (only without EXACT, when the FP32 filter cannot
-// decide; the caller then defers to an exact pass).  Behind every face plane
-// means inside for any closed cell star-shaped about its centre (the segment
-// from the centre to an outside point leaves through a face it ends in front
-// of); for a convex cell, in front of one face means outside.  Other cells
-// take the cone test: find the triangle whose cone from the centre holds q,
-// then q must lie behind that triangle.
-// exit_t (optional): for a cell found outside, a triangle to leave it by: for a
-// convex cell one whose plane q lies in front of, otherwise the one that the
-// ray from the centre to q passes; -1 if none was found.
-// boxcheck = false skips the bounding-box rejection, so that a convex cell
-// the point lies outside of always reports an exit triangle (for walks).
+// The cone test of a cell that need not be convex: 1 when q, in front of the
+// plane of triangle `front`, is inside all the same, else 0 (-1 undecided,
+// without EXACT) with the triangle that the ray from the centre to q passes in
+// *exit_t.  Exactly one cone holds q, mostly that of `front` or one near it, so
+// the search starts there (first binning of 1 048 576 molecules in hexahedra, from
+// the cell's first triangle: 706 us, from `front`: 518).  The filter loads each
+// triangle while the one before it is tested.
 template <bool EXACT>
-__device__ int cell_test(const BinArgs &a, int c, float3 q, const double *p64, int *exit_t = nullptr,
-                         bool boxcheck = true) {
-    if (exit_t) *exit_t = -1;
-    const float *B = a.box32 + 6 * c;
-    const float scale = fmaxf(a.max_local, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
-    const float tol = 1e-5f * scale;
-    if (boxcheck && (q.x < B[0] - tol || q.y < B[1] - tol || q.z < B[2] - tol || q.x > B[3] + tol ||
-                     q.y > B[4] + tol || q.z > B[5] + tol))
-        return 0;
-    const int2 tc = a.tric[c];
-    const int t0 = tc.x, code = tc.y, nt = code & 0xffff;
-    // the face planes: e = n.q - d with |n|_1 = 1 carries at most about
-    // 9 * 2^-24 * scale of rounding (plane, point, three FMAs), far below
-    // the filter's bound; undecided faces go to the exact orientation
-    const float pb = 1e-5f * scale;
-    bool behind = true;
-    int front = t0;                       // the triangle q lies in front of
-    // four planes' loads at a time: one after another, each wait for the cache
-    // (and the early exit behind it) bound this loop
-    for (int tb = t0; behind && tb < t0 + nt; tb += 4) {
-        float4 P[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) P[i] = a.pl32[min(tb + i, t0 + nt - 1)];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int t = tb + i;
-            if (!behind || t >= t0 + nt) break;
-            const float e = fmaf(P[i].z, q.z, fmaf(P[i].y, q.y, fmaf(P[i].x, q.x, -P[i].w)));
-            int s = e > pb ? 1 : (e < -pb ? -1 : 0);
-            if (EXACT && s == 0) {
-                const double *D = a.tri + 9 * t;
-                s = orient_sos_slow(D, D + 3, D + 6, p64);
-            }
-            if (!EXACT && s == 0) return -1;
-            if (s > 0) {
-                behind = false;
-                front = t;
-                if (exit_t) *exit_t = t;
-            }
-        }
-    }
-    if (behind) return 1;
-    if (code >> 16) return 0;
-    if (exit_t) *exit_t = -1;
-    float3 C = ld3f(a.ctr32 + 3 * c);
+__device__ __forceinline__ int cone_test(const BinArgs &a, int c, int t0, int nt, int front, float3 q, float scale,
+                                         const double *p64, int *exit_t) {
+    const float3 C = ld3f(a.ctr32 + 3 * c);
     const double *C64 = a.ctr + 3 * c;
-    // the cone is mostly that of the triangle in front of which q lies, or near
-    // it, so the search starts there (exactly one cone holds q)
-    float N[9];                           // the next triangle, loaded while this one is tested
+    float N[9];
+    if (!EXACT)
 #pragma unroll
-    for (int i = 0; i < 9; ++i) N[i] = a.tri32[9 * front + i];
+        for (int i = 0; i < 9; ++i) N[i] = a.tri32[9 * front + i];
     for (int n = 0, t = front, u; n < nt; ++n, t = u) {
         const double *D = a.tri + 9 * t;
+        if (EXACT)
+#pragma unroll
+            for (int i = 0; i < 9; ++i) N[i] = a.tri32[9 * t + i];
         const float3 x0 = make_float3(N[0], N[1], N[2]), x1 = make_float3(N[3], N[4], N[5]),
                      x2 = make_float3(N[6], N[7], N[8]);
         u = t + 1 < t0 + nt ? t + 1 : t0;
+        if (!EXACT)
 #pragma unroll
-        for (int i = 0; i < 9; ++i) N[i] = a.tri32[9 * u + i];
+            for (int i = 0; i < 9; ++i) N[i] = a.tri32[9 * u + i];
         // p in the cone from C through triangle (x0, x1, x2)?
         int s = orient<EXACT>(C, x0, x1, q, scale, C64, D, D + 3, p64);
         if (!EXACT && s == 0) return -1;
@@ -209,8 +165,104 @@ __device__ int cell_test(const BinArgs &a, int c, float3 q, const double *p64, i
     return 0;
 }
 
+// Not inlined: its registers would be spilled around the searches' plane tests
+// (first binning of 1 048 576 molecules in hexahedra 518 -> 475 us).
+__device__ __noinline__ int cone_exact(const BinArgs &a, int c, int t0, int nt, int front, float3 q, float scale,
+                                       const double *p64) {
+    return cone_test<true>(a, c, t0, nt, front, q, scale, p64, nullptr);
+}
+
+// q (p local to cell c) inside cell c with the SoS tie-break: 1 inside, 0
+// outside, -1 undecided (only without EXACT, when the FP32 filter cannot
+// decide; the caller then defers to an exact pass).  Behind every face plane
+// means inside for any closed cell star-shaped about its centre (the segment
+// from the centre to an outside point leaves through a face it ends in front
+// of); for a convex cell, in front of one face means outside.  Other cells
+// take the cone test: find the triangle whose cone from the centre holds q,
+// then q must lie behind that triangle.
+// exit_t (without EXACT, optional): for a cell found outside, a triangle to
+// leave it by: for a convex cell one whose plane q lies in front of, otherwise
+// the one that the ray from the centre to q passes; -1 if none was found.
+// boxcheck = false skips the bounding-box rejection, so that a convex cell
+// the point lies outside of always reports an exit triangle (for walks).
+// TET: every cell of the mesh has four triangles, so is convex.
+//
+// A test waits for its planes' loads.  The filter mostly starts in the right
+// cell and sees all planes, so it loads four at a time (1 048 576 molecules in
+// hexahedra, cells unchanged: plane by plane 247 us a binning, now 213).  Of a
+// search's candidates most fail at the first or second plane, so it takes them
+// one by one; so do tetrahedra, unrolled, where four planes are the whole cell
+// (8 388 608 molecules in tetrahedra, four at a time against plane by plane:
+// first binning 4 479 -> 2 825 us, after moves of half a diameter 1 113 -> 868).
+template <bool EXACT, bool TET>
+__device__ int cell_test(const BinArgs &a, int c, float3 q, const double *p64, int *exit_t = nullptr,
+                         bool boxcheck = true) {
+    if (exit_t) *exit_t = -1;
+    const float *B = a.box32 + 6 * c;
+    const float scale = fmaxf(a.max_local, fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
+    const float tol = 1e-5f * scale;
+    if (boxcheck && (q.x < B[0] - tol || q.y < B[1] - tol || q.z < B[2] - tol || q.x > B[3] + tol ||
+                     q.y > B[4] + tol || q.z > B[5] + tol))
+        return 0;
+    const int2 tc = a.tric[c];
+    const int t0 = tc.x, code = tc.y, nt = code & 0xffff;
+    // the face planes: e = n.q - d with |n|_1 = 1 carries at most about
+    // 9 * 2^-24 * scale of rounding (plane, point, three FMAs), far below
+    // the filter's bound; undecided faces go to the exact orientation
+    const float pb = 1e-5f * scale;
+    bool behind = true;
+    int front = t0;                       // the triangle q lies in front of
+    auto side = [&](int t, float4 P) {    // of q against triangle t's plane: 1 in front, -1 behind, 0 undecided
+        const float e = fmaf(P.z, q.z, fmaf(P.y, q.y, fmaf(P.x, q.x, -P.w)));
+        int s = e > pb ? 1 : (e < -pb ? -1 : 0);
+        if (EXACT && s == 0) {
+            const double *D = a.tri + 9 * t;
+            s = orient_sos_slow<TET>(D, D + 3, D + 6, p64);
+        }
+        if (s > 0) {
+            behind = false;
+            front = t;
+            if (exit_t) *exit_t = t;
+        }
+        return s;
+    };
+    if (EXACT || TET) {
+        constexpr int kUnroll = TET ? 4 : 1;
+#pragma unroll kUnroll
+        for (int t = t0; t < t0 + nt; ++t) {
+            const int s = side(t, a.pl32[t]);
+            if (!EXACT && s == 0) return -1;
+            if (s > 0) break;
+        }
+    } else {
+        for (int tb = t0; behind && tb < t0 + nt; tb += 4) {
+            float4 P[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) P[i] = a.pl32[min(tb + i, t0 + nt - 1)];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (!behind || tb + i >= t0 + nt) break;
+                if (side(tb + i, P[i]) == 0) return -1;
+            }
+        }
+    }
+    if (behind) return 1;
+    if constexpr (TET) {
+        return 0;
+    } else {
+        if (code >> 16) return 0;
+        if constexpr (EXACT) {
+            return cone_exact(a, c, t0, nt, front, q, scale, p64);
+        } else {
+            if (exit_t) *exit_t = -1;
+            return cone_test<false>(a, c, t0, nt, front, q, scale, p64, exit_t);
+        }
+    }
+}
+
+template <bool TET>
 __device__ __forceinline__ bool cell_contains(const BinArgs &a, int c, float3 q, const double *p64) {
-    return cell_test<true>(a, c, q, p64) == 1;
+    return cell_test<true, TET>(a, c, q, p64) == 1;
 }
 
 // FP64 -> FP32 without the conversion units (on GB300 those share the
@@ -286,6 +338,7 @@ __device__ __forceinline__ void wrapped_position(const BinArgs &a, int64_t k, do
 }
 
 // Search the bucket grid for the cell holding p (skipping cell `skip`).
+template <bool TET>
 __device__ int grid_search(const BinArgs &a, const double *p, int skip) {
     int ib[3];
     for (int d = 0; d < 3; ++d)
@@ -303,12 +356,13 @@ __device__ int grid_search(const BinArgs &a, const double *p, int skip) {
         const float3 q = make_float3(pb.x - (float)(a.orgk[3 * c] - kb[0]) * (1.0f / 1024.0f),
                                      pb.y - (float)(a.orgk[3 * c + 1] - kb[1]) * (1.0f / 1024.0f),
                                      pb.z - (float)(a.orgk[3 * c + 2] - kb[2]) * (1.0f / 1024.0f));
-        if (cell_contains(a, c, q, p)) return c;
+        if (cell_contains<TET>(a, c, q, p)) return c;
     }
     return -1;
 }
 
 // Full search for every molecule (no previous cells).
+template <bool TET>
 __global__ void __launch_bounds__(256) bin_locate(BinArgs a) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int found = -1;
@@ -316,7 +370,7 @@ __global__ void __launch_bounds__(256) bin_locate(BinArgs a) {
         double p[3];
         bool ok;
         wrapped_position(a, k, p, ok);
-        found = ok ? grid_search(a, p, -1) : -1;
+        found = ok ? grid_search<TET>(a, p, -1) : -1;
         a.cell_of[k] = found;
         if (found < 0) {
             a.inv[k] = -1;
@@ -330,53 +384,67 @@ __global__ void __launch_bounds__(256) bin_locate(BinArgs a) {
 // across the face that cell_test names, up to kWalk cells (a visibility walk,
 // as in point location in triangulations); the FP32 filter alone decides each
 // step.  Molecules not found so (the walk met a boundary, an undecided test, or
-// ran out of steps) go to the miss list.  Bound by the latency of the tests'
-// loads: planes come four at a time and triangles one ahead (1 153 768
-// molecules in hexahedra: 134 -> 94 us; one at a time, with an early exit,
-// before; groups of six: 94.5).
-constexpr int kWalk = 8;
+// ran out of steps) go to the miss list.  Bound by the latency of the tests' loads
+// (see cell_test); 1 153 768 molecules of a channel, cells unchanged: plane by
+// plane 338 us a binning, now 240.
+//
+// Who walks.  In tetrahedra, small and convex, all that left.  In other cells a
+// step costs more, a warp waits for the last of its walkers, and the search's
+// warps are many: so only where a warp has at least kWalkers of them (131 072
+// molecules in hexahedra, moves of 0.01 diameter, where few leave: none walk
+// 68 us, all walk 90, now 65; of 0.5 diameter: 145, 109, 79), and none where
+// the search has a warp for every molecule (2 048 molecules, moves of 0.5: all
+// walk 73 us, now 46).  Nor walks a molecule farther from the cell's origin than
+// kFar times the size of the largest cell: it would seldom arrive (256 000
+// molecules in tetrahedra at unrelated positions: 377 us without, 347 with it).
+constexpr int kWalk = 8, kWalkers = 4;
+constexpr float kFar = 4.f;
+template <bool TET>
 __global__ void __launch_bounds__(256) bin_locate_hint(BinArgs a) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool miss = false, undecided = false;
-    int located = -1;
+    bool miss = false, undecided = false, walk = false;
+    int located = -1, c = -1, ex = -1, r = 0;
+    double p[3];
+    // p in a cell's frame without the FP64 pipe: p = ph + pl (split on
+    // the integer units), the cell origin exact in FP32, q = (ph - o) + pl
+    // (at most about 2.2 * 2^-24 of the frame scale off the exact local
+    // point, inside the filter's bound)
+    float ph[3] = {0.f, 0.f, 0.f}, pl[3] = {0.f, 0.f, 0.f};
+    auto loc = [&](int cc) {
+        if (!a.org32) return local_to(a, p, cc);
+        const float *o = a.orgf + 3 * cc;
+        return make_float3((ph[0] - o[0]) + pl[0], (ph[1] - o[1]) + pl[1], (ph[2] - o[2]) + pl[2]);
+    };
     if (k < a.n) {
-        double p[3];
         bool ok;
         wrapped_position(a, k, p, ok);
-        const int h = a.hint[k];
-        if (ok && h >= 0) {
-            // p in a cell's frame without the FP64 pipe: p = ph + pl (split on
-            // the integer units), the cell origin exact in FP32, q = (ph - o) + pl
-            // (at most about 2.2 * 2^-24 of the frame scale off the exact local
-            // point, inside the filter's bound)
-            float ph[3], pl[3];
-            for (int d = 0; d < 3; ++d) split_f64(p[d], ph[d], pl[d]);
-            auto loc = [&](int cc) {
-                if (!a.org32) return local_to(a, p, cc);
-                const float *o = a.orgf + 3 * cc;
-                return make_float3((ph[0] - o[0]) + pl[0], (ph[1] - o[1]) + pl[1], (ph[2] - o[2]) + pl[2]);
-            };
-            int c = h, ex = -1;
-            int r = cell_test<false>(a, c, loc(c), p, &ex, false);
-            undecided = r < 0;
-            for (int step = 0; step < kWalk && r == 0 && ex >= 0; ++step) {
-                c = a.tri_nbr[ex];
-                if (c < 0) break;
-                r = cell_test<false>(a, c, loc(c), p, &ex, false);
-            }
-            if (r == 1) {
-                a.cell_of[k] = c;
-                located = c;
-            } else {
-                miss = true;
-            }
-        } else if (ok) {
-            miss = true;
-        } else {
+        c = a.hint[k];
+        if (!ok) {
             a.cell_of[k] = -1;
             a.inv[k] = -1;
             atomicOr(a.flags, kFlagOutside);
+        } else if (c < 0) {
+            miss = true;
+        } else {
+            for (int d = 0; d < 3; ++d) split_f64(p[d], ph[d], pl[d]);
+            const float3 q = loc(c);
+            r = cell_test<false, TET>(a, c, q, p, &ex, false);
+            undecided = r < 0;
+            miss = r != 1;
+            walk = r == 0 && ex >= 0 && fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))) <= kFar * a.max_local;
         }
+    }
+    if (__popc(__ballot_sync(0xffffffffu, walk)) >= a.walkers && walk) {
+        for (int step = 0; step < kWalk && r == 0 && ex >= 0; ++step) {
+            c = a.tri_nbr[ex];
+            if (c < 0) break;
+            r = cell_test<false, TET>(a, c, loc(c), p, &ex, false);
+        }
+        miss = r != 1;
+    }
+    if (r == 1) {
+        a.cell_of[k] = c;
+        located = c;
     }
     count_located(a, located);
     const unsigned bal = __ballot_sync(0xffffffffu, miss);
@@ -398,11 +466,15 @@ __global__ void __launch_bounds__(256) bin_locate_hint(BinArgs a) {
 // warp takes no more molecules than it must.  Channel of 1 153 768 molecules
 // (a warp per molecule for both before): 103 -> 42 us (with the
 // exact zero for molecules on axis-aligned planes, predicates.cuh).
+template <bool TET>
 __global__ void __launch_bounds__(256) bin_locate_miss(BinArgs a) {
     const int lane = threadIdx.x & 31;
     const int nm = a.miss[0];
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    const int chunk = min(32, (nm + nw - 1) / nw);        // molecules of a warp at a time
+    // molecules of a warp at a time: at most 32, and so many that the warps' rounds
+    // come out even
+    const int rounds = max(1, (nm + 32 * nw - 1) / (32 * nw));
+    const int chunk = max(1, (nm + rounds * nw - 1) / (rounds * nw));
     for (int i0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * chunk; i0 < nm; i0 += nw * chunk) {
         const bool has = lane < chunk && i0 + lane < nm;
         int e = 0, found = -1;
@@ -413,7 +485,7 @@ __global__ void __launch_bounds__(256) bin_locate_miss(BinArgs a) {
                 double p[3];
                 bool ok;
                 wrapped_position(a, k, p, ok);
-                if (cell_contains(a, h, local_to(a, p, h), p)) {
+                if (cell_contains<TET>(a, h, local_to(a, p, h), p)) {
                     found = h;
                     a.cell_of[k] = h;
                     atomicAdd(a.cnt + h, 1);
@@ -438,7 +510,7 @@ __global__ void __launch_bounds__(256) bin_locate_miss(BinArgs a) {
                     bool hit = false;
                     if (j < j1) {
                         c = a.nbr[j];
-                        hit = cell_contains(a, c, local_to(a, p, c), p);
+                        hit = cell_contains<TET>(a, c, local_to(a, p, c), p);
                     }
                     const unsigned bal = __ballot_sync(0xffffffffu, hit);
                     if (bal) {
@@ -459,7 +531,7 @@ __global__ void __launch_bounds__(256) bin_locate_miss(BinArgs a) {
                     bool hit = false;
                     if (ii < i1) {
                         c = a.bkt_cells[ii];
-                        hit = c != h && cell_contains(a, c, local_to(a, p, c), p);
+                        hit = c != h && cell_contains<TET>(a, c, local_to(a, p, c), p);
                     }
                     const unsigned bal = __ballot_sync(0xffffffffu, hit);
                     if (bal) {
@@ -969,16 +1041,25 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     }
     m->bin_clean = false;
     unsigned nb = (unsigned)((n + 255) / 256);
+    const bool tet = m->max_tri == 4;        // closed cells of four triangles
     if (n > 0) {
         // locate every molecule and count the cells' molecules
         if (a.hint) {
             // small systems: small blocks, so that every SM has some of the (latency-bound) warps
             const unsigned lb = n <= 152 * 512 ? 64 : 256;
-            bin_locate_hint<<<(unsigned)((n + lb - 1) / lb), lb, 0, st>>>(a);
-            bin_locate_miss<<<152 * 4, 256, 0, st>>>(a);
+            const unsigned hb = (unsigned)((n + lb - 1) / lb), mb = 152 * 4;
+            a.walkers = tet ? 1 : n <= mb * 8 ? 33 : kWalkers;
+            if (tet) {
+                bin_locate_hint<true><<<hb, lb, 0, st>>>(a);
+                bin_locate_miss<true><<<mb, 256, 0, st>>>(a);
+            } else {
+                bin_locate_hint<false><<<hb, lb, 0, st>>>(a);
+                bin_locate_miss<false><<<mb, 256, 0, st>>>(a);
+            }
             m->launches += 2;
         } else {
-            bin_locate<<<nb, 256, 0, st>>>(a);
+            if (tet) bin_locate<true><<<nb, 256, 0, st>>>(a);
+            else bin_locate<false><<<nb, 256, 0, st>>>(a);
             m->launches += 1;
         }
     }

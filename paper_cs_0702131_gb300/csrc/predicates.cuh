@@ -96,6 +96,12 @@ __host__ __device__ inline void grow_triple(double *e, int &n, double s, const d
 }
 
 // exact sign of det[u; v; w] where u = a - p etc. (rows), FP64 inputs
+//
+// COPY (here and below): kernels that share a function that is not inlined also
+// share the registers that it may use, so point location in tetrahedra, which
+// calls these functions from fewer places, has copies of its own (shared:
+// bin_locate<TET> and bin_locate_miss<TET> spill 120 and 312 bytes, with copies 20 and 104).
+template <int COPY = 0>
 static __host__ __device__ __noinline__ int exact_det3_sign(const double *a, const double *b, const double *c,
                                                    const double *p) {
     double u[3][2], v[3][2], w[3][2];
@@ -117,6 +123,7 @@ static __host__ __device__ __noinline__ int exact_det3_sign(const double *a, con
 }
 
 // exact sign of (b_i - a_i)(c_j - a_j) - (b_j - a_j)(c_i - a_i)
+template <int COPY = 0>
 static __device__ __noinline__ int exact_det2_sign(const double *a, const double *b, const double *c, int i, int j) {
     {
         // FP64 first: differences and products carry a few 2^-53 of their
@@ -153,6 +160,7 @@ static __device__ __noinline__ int exact_det2_sign(const double *a, const double
 
 // --------------------------------------------------------------- the predicate
 // FP64 stage and exact stage of the perturbed orientation sign (FP64 inputs).
+template <int COPY = 0>
 static __device__ __noinline__ int orient_sos_slow(const double *a, const double *b, const double *c, const double *p) {
     double u[3], v[3], w[3];
     for (int d = 0; d < 3; ++d) {
@@ -170,14 +178,14 @@ static __device__ __noinline__ int orient_sos_slow(const double *a, const double
     else if ((u[0] == 0.0 && v[0] == 0.0 && w[0] == 0.0) || (u[1] == 0.0 && v[1] == 0.0 && w[1] == 0.0) ||
              (u[2] == 0.0 && v[2] == 0.0 && w[2] == 0.0))
         s = 0;               // p on the triangle's axis-aligned plane (walls on lattice planes): exactly zero
-    else s = exact_det3_sign(a, b, c, p);
+    else s = exact_det3_sign<COPY>(a, b, c, p);
     if (s != 0) return -s;   // O = -det[a-p; b-p; c-p]
     // p on the plane: N_x, N_y, N_z of N = (b - a) x (c - a), exactly
-    int nx = exact_det2_sign(a, b, c, 1, 2);
+    int nx = exact_det2_sign<COPY>(a, b, c, 1, 2);
     if (nx) return nx;
-    int ny = exact_det2_sign(a, b, c, 2, 0);
+    int ny = exact_det2_sign<COPY>(a, b, c, 2, 0);
     if (ny) return ny;
-    return exact_det2_sign(a, b, c, 0, 1);
+    return exact_det2_sign<COPY>(a, b, c, 0, 1);
 }
 
 // FP32 filter on coordinates local to a common origin.  The local copies
