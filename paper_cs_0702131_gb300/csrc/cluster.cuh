@@ -1,4 +1,4 @@
-// Building blocks of the queued cluster kernels: a warp takes one cluster of
+// Building blocks of the FP64 cluster kernels (pair64.cu): a warp takes one cluster of
 // cells (or one of `parts` shares of its candidates), collects the partner
 // molecules that survive the cull against the cluster's box into a buffer in
 // shared memory (cl_fill), tests them against the cluster's molecules with
@@ -92,8 +92,8 @@ __device__ __forceinline__ void cl_box_of(const PairArgs &a, ClShare<CAP> &w, in
 // the cluster's candidates are used up (false): A's own molecules (their
 // packed words carry kSameBit and the cell label), then the molecules of its
 // partner runs, moved into A's frame and culled against A's box.  Group g of
-// 32 candidates belongs to share g mod parts.  store(slot, l, o, xh): l the
-// binned index, o the entry of ed (own molecules: -1), xh position and word.
+// 32 candidates belongs to share g mod parts.  store(slot, l, xh): l the
+// binned index, xh position and word.  Halo molecules (portion mode) are not marked.
 template <int CAP, class Store>
 __device__ __forceinline__ bool cl_fill(const PairArgs &a, const ClKArgs &c, ClShare<CAP> &w, ClCursor &q, int &nq,
                                         float rcut2, int part, int parts, int lane, Store store) {
@@ -106,8 +106,8 @@ __device__ __forceinline__ bool cl_fill(const PairArgs &a, const ClKArgs &c, ClS
                 if (alive) {
                     float4 x = a.xloc[k];
                     const int w0 = __float_as_int(x.w), lab = __float_as_int(c.xlo[k].w) & 15;
-                    x.w = __int_as_float((w0 & kSpBits) | kSameBit | (lab << 5) | ((w0 & kGhostBit) ? kGhostW : 0));
-                    store(nq + lane, k, -1, x);
+                    x.w = __int_as_float((w0 & kSpBits) | kSameBit | (lab << 5));
+                    store(nq + lane, k, x);
                 }
                 nq += min(32, q.s1 - q.own);
             }
@@ -121,9 +121,9 @@ __device__ __forceinline__ bool cl_fill(const PairArgs &a, const ClKArgs &c, ClS
                 const int p = q.p0 + lane;
                 bool alive = false;
                 float4 xh = make_float4(0.f, 0.f, 0.f, 0.f);
-                int l = 0, o = 0;
+                int l = 0;
                 if (p < q.total) {
-                    o = base + __popc(M & le);
+                    const int o = base + __popc(M & le);
                     l = p + w.eb[o];
                     const float4 dh = w.ed[o], x = a.xloc[l];
                     xh = make_float4(x.x + dh.x, x.y + dh.y, x.z + dh.z, 0.f);
@@ -133,11 +133,10 @@ __device__ __forceinline__ bool cl_fill(const PairArgs &a, const ClKArgs &c, ClS
                     alive = dx * dx + dy * dy + dz * dz <= rcut2;
                     const int code = __float_as_int(dh.w) >> 12;
                     const int w0 = __float_as_int(x.w);
-                    xh.w = __int_as_float((w0 & kSpBits) | (code != 0 ? kImgBit : 0) | (code << 9) |
-                                          ((w0 & kGhostBit) ? kGhostW : 0));
+                    xh.w = __int_as_float((w0 & kSpBits) | (code != 0 ? kImgBit : 0) | (code << 9));
                 }
                 const unsigned bal = __ballot_sync(FULL, alive);
-                if (alive) store(nq + __popc(bal & lt), l, o, xh);
+                if (alive) store(nq + __popc(bal & lt), l, xh);
                 nq += __popc(bal);
                 q.culls += (unsigned)min(32, q.total - q.p0);
             }
@@ -193,7 +192,7 @@ __device__ __forceinline__ int cl_load_tile(const PairArgs &a, const ClKArgs &c,
         if (lane < ni) {
             x = a.xloc[k0 + lane];
             const int w0 = __float_as_int(x.w), lab = __float_as_int(c.xlo[k0 + lane].w) & 15;
-            w.tw[lane] = (w0 & kSpBits) | (lab << 5) | ((w0 & kGhostBit) ? kGhostW : 0);
+            w.tw[lane] = (w0 & kSpBits) | (lab << 5);
             atomicOr(&w.cellm[lab], 1u << (ne - 1 - lane));
         }
         float *xy = (float *)&w.txy[lane >> 1];

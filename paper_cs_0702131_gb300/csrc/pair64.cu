@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kW64 * 32) pair64c(PairArgs a, ClKArgs c, Tab6
         const int ntile = (nA + kTile - 1) / kTile, wtile = (nA + ntile - 1) / ntile;
         for (bool more = true; more;) {
             int nq = 0;
-            more = cl_fill(a, c, w, q, nq, rcut2, part, parts, lane, [&](int slot, int l, int, float4 xh) {
+            more = cl_fill(a, c, w, q, nq, rcut2, part, parts, lane, [&](int slot, int l, float4 xh) {
                 w.sh[slot] = xh;
                 w.sl[slot] = l;
             });
