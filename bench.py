@@ -34,7 +34,9 @@ METRIC = "LJ pair interactions/s within rc (FP32 vs FP64 on same GB300) at state
 UNIT = "pairs/s"
 FLOPS_EVAL, FLOPS_WITHIN = 8, 32     # the method's work: flops per AICA-evaluated pair (distance test)
                                      # and per pair within rc (force, energy, virial)
-FLOPS64_EVAL, FLOPS64_WITHIN = 14, 35  # FP64 path: (x_k - x_l) - n.L and r^2 unfused; pair body
+FLOPS64_EVAL, FLOPS64_WITHIN = 14, 35  # FP64 cell kernel: (x_k - x_l) - n.L and r^2 unfused; pair body
+FLOPS64_CLUSTER = 36                 # FP64 cluster kernel, per pair within rc, in 22 instructions: separation 3,
+                                     # r^2 5, 1/r^2 6, powers and force factor 6, energy 4, both forces 12
 BIN_BYTES = 84                       # binning: pos 24 + species 4 + previous cell 4 read; cell, order,
                                      # inverse 4 each + float4 16 + FP64 copy 24 written, per molecule
 FORCE_TOL = {"fp32": 1e-5, "fp64": 1e-12}
@@ -310,14 +312,15 @@ def run_ours(args):
             # the cluster kernel tests in FP32 and forms only the pairs within rc in FP64
             # (halo molecules: the cell kernel, which tests in FP64)
             cl64 = mesh.get_option("cluster_path") == 1 and int(os.environ.get("WORLD_SIZE", "1")) == 1
-            tests64 = w64 if cl64 else int(stats64[0])
-            fl64 = FLOPS64_EVAL * tests64 + FLOPS64_WITHIN * w64
+            tests64 = int(stats64[0])
+            fl64 = FLOPS64_CLUSTER * w64 if cl64 else FLOPS64_EVAL * tests64 + FLOPS64_WITHIN * w64
             fp64["roofline"] = {"kernel": "pair64c" if cl64 else "pair_fwd64", "bound": "alu",
                                 "achieved": round(fl64 / (k64 * 1e-3) / 1e12, 4),
                                 "peak": round(peak64, 4), "unit": "TFLOP/s",
                                 "frac": round(fl64 / (k64 * 1e-3) / 1e12 / peak64, 4), "kernel_ms": round(k64, 4),
                                 "peak_basis": "measured FP64 FMA rate of this GPU (aica_probe_fma_rate)",
-                                "flop_model": (f"{FLOPS64_EVAL} per FP64 separation and r^2 ({tests64}) + "
+                                "flop_model": (f"{FLOPS64_CLUSTER} per within-rc pair; FP32 tests not counted" if cl64 else
+                                               f"{FLOPS64_EVAL} per FP64 separation and r^2 ({tests64}) + "
                                                f"{FLOPS64_WITHIN} per within-rc pair; FP32 tests not counted")}
 
     out = None
