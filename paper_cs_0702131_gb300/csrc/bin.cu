@@ -943,8 +943,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int C = (int)m->n_cells;
-    const bool runs = really_ran(st);
-    if (!runs) m->captured = true;
+    if (m->deferred && !really_ran(st)) m->captured = true;      // (a checked call cannot be captured: it waits)
     m->launches = 0;
     m->binned = false;
     if (n > m->cap_mol) {
@@ -1086,7 +1085,7 @@ extern "C" aica_status aica_bin_molecules(aica_mesh *m, const double *pos, const
     m->n_mol_prev = n;
     m->hint_valid = true;
     AICA_CUDA(cudaGetLastError());
-    m->bin_clean = was_clean || runs;
+    m->bin_clean = was_clean || really_ran(st);
     if (cell_of && n) AICA_CUDA(cudaMemcpyAsync(cell_of, a.cell_of, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (order && n) AICA_CUDA(cudaMemcpyAsync(order, m->order.p, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     if (cell_off) AICA_CUDA(cudaMemcpyAsync(cell_off, off, sizeof(int) * (C + 1), cudaMemcpyDeviceToDevice, st));
