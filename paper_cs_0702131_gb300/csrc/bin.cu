@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(256) bin_locate_hint(BinArgs a) {
 // parallel, then the cells of the molecule's bucket.  Exact predicates make at
 // most one cell hold the point.  Bound by the latency of the exact tests, so a
 // warp takes no more molecules than it must.  Channel of 1 153 768 molecules
-// (a warp per molecule for both before): 103 -> 42 us (with the
+// (a warp per molecule for both before): 103 -> 39 us (with the
 // exact zero for molecules on axis-aligned planes, predicates.cuh).
 template <bool TET>
 __global__ void __launch_bounds__(256) bin_locate_miss(BinArgs a) {

@@ -7,9 +7,9 @@
 // (cluster.cuh), only the pairs within rc reach the FP64 body, and a lane
 // always has one of them (the survivors are dealt out by their pair counts).
 // A separation is formed as the all-pairs definition rounds it, three FP64
-// subtractions (six for periodic images); 1/r^2 starts from the FP32 reciprocal and takes one cubic
-// step (e = 1 - r^2 y; y + y (e + e^2), from a relative error below 2^-21 to
-// below 2^-62 before the last rounding); conversions are done on the bit
+// subtractions (six for periodic images); 1/r^2 starts from the FP32 reciprocal and takes one step
+// of the hyperpower iteration of order three (e = 1 - r^2 y; y + y (e + e^2), from a
+// relative error below 2^-21 to below 2^-62 before the last rounding); conversions are done on the bit
 // patterns, which would otherwise run on the FP64 pipe too; and the virial is
 // the sum of x (x) F over the forces a warp hands out (x in the cluster's
 // frame; each pair adds f and -f, so the origin cancels) instead of six products

@@ -19,9 +19,8 @@ BOX = dict(L=L, periodic=np.array([1, 1, 1], np.int32))
 
 
 def _mixed(rng):
-    """Every third hexahedron of a jittered grid as six tetrahedra, if its
-    faces agree with its neighbours': here the tetrahedra fill whole layers, so
-    the mesh is two stacks glued at a plane of the box."""
+    """Two stacks, one of tetrahedra and one of hexahedra, that meet at z = 7.5
+    without being neighbours: a walk ends there."""
     lo, hi = np.zeros(3), L.copy()
     hi[2] = 7.5
     a = synth.hex_mesh((6, 6, 3), lo, hi, 0.15, rng, tets=True)
